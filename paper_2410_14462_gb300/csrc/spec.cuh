@@ -213,6 +213,81 @@ __device__ __forceinline__ float alpha_at_nb(float mx, float my, float ca, float
     return pw > 0.0f ? 0.0f : al;
 }
 
+// Two float32 values in one register pair.  Blackwell's packed instructions
+// round each half like the scalar ones, at half the instruction count.
+// Unlike the scalar forms, the assembler contracts mul.rn.f32x2 and
+// add.rn.f32x2 into one fused operation (measured: every sum of a product
+// differed from the twice-rounded one), so a sum whose roundings must stay
+// apart is f2_sum: a fused a * one + b with a `one` that is only known at run
+// time.
+struct F2 {
+    uint64_t v;
+};
+__device__ __forceinline__ F2 f2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_get(F2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+__device__ __forceinline__ F2 f2_sum(F2 a, F2 b, F2 one) { return f2_fma(a, one, b); }
+
+// alpha_at of one Gaussian at two pixel centres, rounding for rounding: the
+// Gaussian's parameters and the pixel's y come in both halves, the pixel
+// centres negated (exact).  The exponent is carried negated, m = -pw (every
+// step's rounding is symmetric), so that 0 <= m <= 87 is one unsigned
+// comparison of its bits (m is never -0).  exp_neg's integer part is rounded by
+// adding and subtracting 1.5 * 2^23 (round to nearest even, as rintf), and 2^n
+// goes into the exponent field by an integer add (exact where the result is
+// normal; elsewhere alpha is under 1/255 and skipped).
+// dx = mx - px and adx2 = ca (dx dx) are the caller's (the same for every row).
+__device__ __forceinline__ float2 alpha_at_x2(F2 dx, F2 adx2, F2 my, F2 cb, F2 cc, F2 op, F2 npy, F2 one) {
+    const F2 dy = f2_add(my, npy);
+    const F2 s = f2_sum(adx2, f2_mul(cc, f2_mul(dy, dy)), one);
+    // (0.5 s is exact, so that product may be fused)
+    const F2 m = f2_fma(f2(0.5f, 0.5f), s, f2_mul(cb, f2_mul(dx, dy)));
+    constexpr float kRound = 12582912.0f;
+    const F2 t = f2_sum(f2_mul(m, f2(-0x1.715476p+0f, -0x1.715476p+0f)), f2(kRound, kRound), one);
+    const F2 n = f2_add(t, f2(-kRound, -kRound));
+    F2 u = f2_fma(n, f2(0x1.62e430p-1f, 0x1.62e430p-1f), m);   // u = -r
+    u = f2_fma(n, f2(-0x1.05c610p-29f, -0x1.05c610p-29f), u);
+    // the polynomial in r = -u, every second partial value negated
+    F2 p = f2_fma(f2(-0x1.a01a02p-13f, -0x1.a01a02p-13f), u, f2(0x1.6c16c2p-10f, 0x1.6c16c2p-10f));
+    p = f2_fma(p, u, f2(-0x1.111112p-7f, -0x1.111112p-7f));
+    p = f2_fma(p, u, f2(0x1.555556p-5f, 0x1.555556p-5f));
+    p = f2_fma(p, u, f2(-0x1.555556p-3f, -0x1.555556p-3f));
+    p = f2_fma(p, u, f2(0.5f, 0.5f));
+    p = f2_fma(p, u, f2(-1.0f, -1.0f));
+    p = f2_fma(p, u, f2(1.0f, 1.0f));
+    const float2 tt = f2_get(t), pp = f2_get(p), mm = f2_get(m);
+    const float ex = __uint_as_float((__float_as_uint(tt.x) << 23) + __float_as_uint(pp.x));
+    const float ey = __uint_as_float((__float_as_uint(tt.y) << 23) + __float_as_uint(pp.y));
+    const float2 al = f2_get(f2_mul(op, f2(ex, ey)));
+    const float ax = fminf(al.x, kAlphaMax), ay = fminf(al.y, kAlphaMax);
+    const uint32_t lim = 0x42ae0000u;   // 87
+    return make_float2(__float_as_uint(mm.x) <= lim && ax >= kAlphaMin ? ax : 0.0f,
+                       __float_as_uint(mm.y) <= lim && ay >= kAlphaMin ? ay : 0.0f);
+}
+
 // Conservative test: can a projected Gaussian reach alpha >= 1/255 at some
 // pixel centre of the rectangle [xa, xb] x [ya, yb]?  It can only if
 //   Q_min = min over the rectangle of  a dx^2 + 2 b dx dy + c dy^2  <=  2 ln(255 o)
@@ -380,6 +455,35 @@ __device__ __forceinline__ uint32_t block_mask_fast(float mx, float my, float a,
         const float xl = mx - hi - epsx, xr = mx - lo + epsx;
         if (xr >= xt && xl <= xt + 7.0f) m |= 1u << (2 * k);
         if (xr >= xt + 8.0f && xl <= xt + 15.0f) m |= 1u << (2 * k + 1);
+    }
+    return m;
+}
+
+// The same test per 16x4 band of the tile (bit k: rows 4 k .. 4 k + 3), for
+// the weights pass, whose warps take a tile band by band.
+__device__ __forceinline__ uint32_t band_mask_fast(float mx, float my, float a, float b, float c, float op, int tx,
+                                                   int ty) {
+    if (op < kAlphaMin) return 0u;
+    const float thr = 2.0f * __logf(255.0f * op) * 1.001f + 1e-3f;
+    const float det = a * c - b * b;
+    if (!(det > 0.0f) || !(thr > 0.0f) || !(a > 0.0f) || !(c > 0.0f)) return 0xfu;
+    const float inv_a = __fdividef(1.0f, a), inv_det = __fdividef(1.0f, det);
+    const float umax = sqrt_approx(thr * c * inv_det);
+    const float wmax = sqrt_approx(thr * a * inv_det) * 1.0002f + 0.05f;
+    const float ws = -b * umax * __fdividef(1.0f, c);
+    const float thra = thr * a;
+    const float epsx = 2e-3f * (umax + 1.0f) + 0.05f;
+    const float xt = (float)(tx * kTile) + 0.5f, yt = (float)(ty * kTile) + 0.5f;
+    uint32_t m = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float ylo = yt + (float)(4 * k);
+        const float w0 = fmaxf(my - (ylo + 3.0f), -wmax), w1 = fminf(my - ylo, wmax);
+        if (w0 > w1) continue;
+        const float s0 = sqrt_approx(thra - det * w0 * w0), s1 = sqrt_approx(thra - det * w1 * w1);
+        const float hi = (ws >= w0 && ws <= w1) ? umax : fmaxf((-b * w0 + s0) * inv_a, (-b * w1 + s1) * inv_a);
+        const float lo = (-ws >= w0 && -ws <= w1) ? -umax : fminf((-b * w0 - s0) * inv_a, (-b * w1 - s1) * inv_a);
+        if (mx - lo + epsx >= xt && mx - hi - epsx <= xt + 15.0f) m |= 1u << k;
     }
     return m;
 }

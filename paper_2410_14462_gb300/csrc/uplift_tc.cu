@@ -12,21 +12,15 @@
 //
 // Two kernels per chunk of views:
 //
-//  k_weights (CUDA cores, one CTA of 8 warps per (view, tile), several CTAs
-//  per SM): walks the tile's depth-ordered list in batches of 32 Gaussians
-//  (float32 rules of Eq. 1: alpha, 1/255 skip, 1e-4 stop), one 8x4 pixel block
-//  per warp.  Warp 0 gathers the batches' projected records (from the
-//  depth-ordered record array, by the ranks the list holds) with cp.async
-//  kRing - 1 batches ahead, and computes each entry's 8x4 block mask once its
-//  record has landed (the next batch's masks after its own compositing of
-//  the current one); only the batches the walk reaches are gathered.  The
-//  batch's weights go to 32 staging rows in shared memory; the Gaussians with
-//  a non-zero weight somewhere in the tile are then appended, as dense
-//  bfloat16 rows of 256 pixels, to the tile's "chunks" of 128 rows in global
-//  memory (chunk ids from an atomic counter; row count, Gaussian ids, den and
-//  the tile's next chunk recorded per chunk, the first chunk per tile).  For
-//  d <= 4 (k_weights<NT, true>) each new row is instead dotted with the
-//  tile's features and added to num and den on the spot.
+//  k_weights (CUDA cores, one warp per (view, tile), see the kernel): walks the
+//  tile's depth-ordered list (float32 rules of Eq. 1: alpha, 1/255 skip, 1e-4
+//  stop) with two neighbouring pixels per lane in packed float32 arithmetic,
+//  and appends the Gaussians with a non-zero weight somewhere in the tile, as
+//  dense bfloat16 rows of 256 pixels, to the tile's "chunks" of 128 rows in
+//  global memory (chunk ids from an atomic counter; row count, Gaussian ids,
+//  den and the tile's next chunk recorded per chunk, the first chunk per
+//  tile).  For d <= 4 each new row is instead dotted with the tile's features
+//  in registers and added to num and den.
 //
 //  k_aggregate_tc (one persistent CTA per SM, warp-specialised, tiles taken
 //  round-robin with each tile's chunks back to back).  Per chunk the K loop is
@@ -74,8 +68,6 @@ namespace {
 
 using namespace tc;
 
-constexpr int kTcBatch = 32;                           // Gaussians composited per step
-constexpr int kRing = 8;                               // list-record batches in flight
 constexpr int kCRows = 128;                            // rows per chunk (MMA M)
 constexpr int kRowBytes = 256 * 2;                     // one row: 256 pixels, bfloat16
 constexpr uint32_t kChunkBytes = kCRows * kRowBytes;   // 64 KB per term
@@ -110,54 +102,14 @@ struct WeightsArgs {
     // direct accumulation (k_weights<NT, true>, few channels): each new row's
     // sum_p w F[p, c] and its den go straight into the view's num and den
     // (atomic adds); no weight rows, chunks or plan are written
-    int direct_d;           // channels, 1 .. kDirectMaxD
     int num_stride;         // floats per Gaussian in num
-    const void* feats;      // [.., H, W, direct_d] float32 or bfloat16, views at views.fview
-    int feat_bf16;
+    const void* feats;      // [.., H, W, DD] float32 (NT = 2) or bfloat16, views at views.fview
+    float2 one;             // {1, 1}: see f2_sum
     AggViews views;
 };
 
 constexpr int kDirectMaxD = 4;
-
-template <int NT>
-struct WeightsSmemBase {
-    alignas(16) PairRec rec[kRing][kTcBatch];
-    alignas(16) uint8_t stage[NT][kTcBatch * kRowBytes];   // [term][j][256 pixels]
-    uint32_t rowmask[2];
-    int cur_chunk, cur_start, next_chunk;
-};
-template <int NT, bool DIRECT>
-struct WeightsSmem : WeightsSmemBase<NT> {};
-template <int NT>
-struct WeightsSmem<NT, true> : WeightsSmemBase<NT> {
-    alignas(16) float feat[kDirectMaxD][256];   // the tile's features by channel and pixel (0 off the image)
-};
-
-// A weight row's contribution to den, from its 256 bfloat16 values (8 per
-// lane, packed in wv), summed over the warp: the sum of the term's values, or
-// with count_den the number of non-zero weights (counted on term 0; a weight
-// w > 0 is at least 1/255 * 1e-4, far above the smallest bfloat16).
-__device__ __forceinline__ float lane_den(const uint32_t* wv, int count_den, int term) {
-    float s = 0.f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (count_den)
-            s += term == 0 ? (float)((wv[k] & 0xffffu) != 0u) + (float)((wv[k] >> 16) != 0u) : 0.f;
-        else
-            s += __uint_as_float(wv[k] << 16) + __uint_as_float(wv[k] & 0xffff0000u);
-    }
-    return s;
-}
-
-__device__ __forceinline__ float warp_sum(float s) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
-
-__device__ __forceinline__ float row_den(const uint32_t* wv, int count_den, int term) {
-    return warp_sum(lane_den(wv, count_den, term));
-}
+constexpr int kBandItems = 152 * 16;
 
 __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int rows, int next) {
     if (c >= 0 && c < a.cap) {
@@ -166,293 +118,290 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
     }
 }
 
-template <int NT, bool DIRECT>
-__global__ void __launch_bounds__(256, 5) k_weights(const __grid_constant__ WeightsArgs a) {
-    __shared__ WeightsSmem<NT, DIRECT> S;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// The weights of one (view, tile), a warp per tile (NB = 4) or per 16x4 band of
+// it (NB = 1): band b is the tile's pixels 64 b .. 64 b + 63, lane l holds
+// pixels 64 b + 2 l and + 1.
+//   DD = 0: weight rows; DD = 1 .. 4: direct accumulation of DD channels.
+//
+// Bound: instruction issue (half FMA pipe, half ALU), with the launch's tail
+// (0.25 to 0.4 ms until the longest tiles end) next to it; a paper-scale tile
+// walks about 210 of its 2200 entries, 550 (entry, band) pairs.  Hence
+//  - two pixels per lane: Blackwell's packed float32 instructions halve the
+//    arithmetic's issue slots (25 packed operations per 64 pixels);
+//  - a warp owns the tile, so nothing waits at a block barrier and a row of
+//    256 pixels leaves as one coalesced 128-byte store per band and term,
+//    without staging; entries are skipped per band (a bit mask per entry);
+//  - a row's lane sums wait in shared memory and are added up with one lane per
+//    row (2 instructions a row where a shuffle reduction takes 10), and so are
+//    the few channels of the direct form, whose atomics then come 32 at once;
+//  - where both bands of a pair are reached they are computed side by side, for
+//    the long tiles that end a launch.
+// 28 warps per SM (72 registers): 20, 24 and 32 measured 2.95, 2.78 and 2.65 ms
+// against 2.62.  20 paper-scale views (1M Gaussians, 980x546, float32): 4.30 ->
+// 2.62 ms against one block of 8 warps per tile with a weight row staged in
+// shared memory; 48 views of 640x480, bfloat16 rows: 6.40 -> 4.0 ms; 60 views
+// of 640x480, 3 channels direct: 6.81 -> 3.75 ms.
+template <int NT, int DD, int NB>
+__global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_constant__ WeightsArgs a) {
+    constexpr bool kDirect = DD > 0;
+    constexpr int kVals = kDirect ? DD + 1 : 1;   // sums per row
+    constexpr int kRowBuf = 32 / kVals;           // rows whose lane sums are kept
+    constexpr uint32_t kAll = 0xffffffffu;
+    __shared__ float4 s_rec[32][3];               // the batch's records, every value twice
+    __shared__ float s_part[32 * 33];             // [row][sum][lane]
+    __shared__ uint32_t s_gid[kRowBuf];
+    const int lane = threadIdx.x;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    const int item = blockIdx.x;
+    const int item = NB == 4 ? (int)blockIdx.x : (int)(blockIdx.x >> 2);
+    const int band0 = NB == 4 ? 0 : (int)(blockIdx.x & 3u);
+    const uint2 range = a.ranges[item];
+    if (range.x >= range.y) return;
     const int v = item / a.ntiles, tile = item - v * a.ntiles;
     const int tx = tile % a.TX, ty = tile / a.TX;
-    const uint2 range = a.ranges[item];
-    const uint32_t nb = (range.y - range.x + kTcBatch - 1) / kTcBatch;
-    if (nb == 0) return;
-    // warp w covers the 8x4 pixel block ((w & 1) * 8, (w >> 1) * 4) of the tile
-    const int lx = (warp & 1) * 8 + (lane & 7), ly = (warp >> 1) * 4 + (lane >> 3);
-    const int pix = ly * kTile + lx;
-    const int px = tx * kTile + lx, py = ty * kTile + ly;
-    const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
-
-    if (tid == 0) {
-        S.rowmask[0] = 0u;
-        S.rowmask[1] = 0u;
-        S.cur_chunk = -1;
-        S.cur_start = 0;
-        S.next_chunk = -1;
-    }
-    for (int e = tid; e < (int)(NT * kTcBatch * kRowBytes / 16); e += 256)
-        reinterpret_cast<uint4*>(&S.stage[0][0])[e] = make_uint4(0u, 0u, 0u, 0u);
-    if constexpr (DIRECT) {
-        // this thread's pixel's channels (zero off the image: no weight there)
-        const bool in_img = px < a.width && py < a.height;
-        const size_t pidx = ((size_t)a.views.fview[v] * a.height + (in_img ? py : 0)) * a.width + (in_img ? px : 0);
+    const int px = tx * kTile + 2 * (lane & 7), py = ty * kTile + 4 * band0 + (lane >> 3);
+    const F2 npx = f2(-((float)px + 0.5f), -((float)px + 1.5f));
+    const F2 one = f2(a.one.x, a.one.y);
+    const bool count = a.count_den != 0;
+    F2 npy[NB];
+    float T[NB][2];   // transmittance; 0 once the pixel is done
 #pragma unroll
-        for (int c = 0; c < kDirectMaxD; ++c) {
-            float x = 0.f;
-            if (in_img && c < a.direct_d)
-                x = a.feat_bf16
-                        ? __bfloat162float(static_cast<const __nv_bfloat16*>(a.feats)[pidx * a.direct_d + c])
-                        : static_cast<const float*>(a.feats)[pidx * a.direct_d + c];
-            S.feat[c][pix] = x;
+    for (int b = 0; b < NB; ++b) {
+        const float y = -((float)(py + 4 * b) + 0.5f);
+        npy[b] = f2(y, y);
+        T[b][0] = px < a.width && py + 4 * b < a.height ? 1.0f : 0.0f;
+        T[b][1] = px + 1 < a.width && py + 4 * b < a.height ? 1.0f : 0.0f;
+    }
+    F2 feat[kDirect ? DD : 1][NB];
+    if constexpr (kDirect) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const size_t p = ((size_t)a.views.fview[v] * a.height + (py + 4 * b)) * a.width + px;
+#pragma unroll
+            for (int c = 0; c < DD; ++c) {
+                float x[2] = {0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    if (T[b][q] > 0.f)
+                        x[q] = NT == 1 ? __bfloat162float(static_cast<const __nv_bfloat16*>(a.feats)[(p + q) * DD + c])
+                                       : static_cast<const float*>(a.feats)[(p + q) * DD + c];
+                feat[c][b] = f2(x[0], x[1]);
+            }
         }
     }
-    __syncthreads();
 
-    // batch k of the list goes to ring slot k % kRing.  Warp 0, lane j gathers
-    // entry j of a batch (two 16-byte cp.async of its 32-byte record) and
-    // commits one cp.async group per batch, empty past the list's end, so
-    // that "at most kRing - 2 groups pending" always means "batch k landed".
-    // The rank of the batch after next is loaded one iteration early, so the
-    // gather does not wait on it.
+    // entry j of batch k is lane j's: its record is loaded one batch ahead, its
+    // rank two
     const PairRec* vrec = a.srec + (int64_t)v * a.npad;
     auto rank_of = [&](uint32_t k) -> uint32_t {
-        const uint32_t e = range.x + k * kTcBatch + (uint32_t)lane;
-        return (k < nb && e < range.y) ? a.rank[e] : 0xffffffffu;
+        const uint32_t e = range.x + 32u * k + (uint32_t)lane;
+        return e < range.y ? a.rank[e] : kAll;
     };
-    auto issue_records = [&](uint32_t k, uint32_t rk) {
-        if (warp == 0) {
-            if (rk != 0xffffffffu) {
-                PairRec* dst = &S.rec[k % kRing][lane];
-                cp_async_16(dst, vrec + rk);
-                cp_async_16(reinterpret_cast<uint8_t*>(dst) + 16, reinterpret_cast<const uint8_t*>(vrec + rk) + 16);
-            }
-            cp_async_commit();
-        }
+    float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
+    auto load_record = [&](uint32_t rk) {
+        if (rk == kAll) return;
+        const float4* p = reinterpret_cast<const float4*>(vrec + rk);
+        ra = p[0];
+        rb = p[1];
     };
-    uint32_t next_rank = 0xffffffffu;   // warp 0: rank of batch k + kRing - 1 at iteration k
-    // warp 0, lane j: entry j of batch k has landed; its block mask.  Batch 0's
-    // is computed here, batch k + 1's after warp 0 has composited batch k (off
-    // the path of the other warps, which are still compositing batch k)
-    auto mask_batch = [&](uint32_t k) {
-        cp_async_wait<kRing - 2>();
-        if (k < nb && range.x + k * kTcBatch + (uint32_t)lane < range.y) {
-            PairRec& r = S.rec[k % kRing][lane];
-            r.mask = block_mask_fast(r.mx, r.my, r.ca, r.cb, r.cc, r.op, tx, ty);
-        }
-    };
-    if (warp == 0) {
-        for (uint32_t k = 0; k + 1 < (uint32_t)kRing; ++k) issue_records(k, rank_of(k));
-        next_rank = rank_of(kRing - 1);
-        mask_batch(0);
-    }
+    load_record(rank_of(0));
+    uint32_t next_rank = rank_of(1);
 
-    float T = 1.0f;
-    bool done = !(px < a.width && py < a.height);
-    int nrows = 0;   // rows of this tile written so far
-    int buf = 0;
-    for (uint32_t k = 0; k < nb; ++k, buf ^= 1) {
-        const uint32_t slot = k % kRing;
-        if (__syncthreads_count(!done) == 0) break;
-        // every thread is past batch k-1: its slot takes batch k + kRing - 1
-        if (warp == 0) {
-            issue_records(k + kRing - 1, next_rank);
-            next_rank = rank_of(k + kRing);
+    uint32_t alive = 0u;   // bands with a pixel that is not done
+#pragma unroll
+    for (int b = 0; b < NB; ++b) alive |= __any_sync(kAll, T[b][0] + T[b][1] > 0.f) ? 1u << b : 0u;
+
+    int cur = -1, local = kCRows;   // the tile's chunk being filled and its rows so far
+    bool keep = false;
+    uint8_t *d1 = nullptr, *d2 = nullptr;
+    int nbuf = 0;   // rows in s_part
+    const uint32_t nb = (range.y - range.x + 31u) / 32u;
+    float* const vnum = kDirect ? a.views.num[v] : nullptr;
+    float* const vden = kDirect ? a.views.den[v] : nullptr;
+    // sum `i` of the kept rows over the lanes
+    auto lane_sum = [&](int i) {
+        const float* p = s_part + 33 * i;
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int l = 0; l < 32; l += 4) {
+            s[0] += p[l];
+            s[1] += p[l + 1];
+            s[2] += p[l + 2];
+            s[3] += p[l + 3];
         }
-        if (!DIRECT && tid == 0) {
-            // rows [nrows, nrows + 32) must have chunks; a chunk filled to
-            // exactly 128 rows may not have its successor yet
-            if (nrows >= S.cur_start + kCRows) {
-                if (S.next_chunk < 0) S.next_chunk = atomicAdd(a.chunk_counter, 1);
-                finish_chunk(a, S.cur_chunk, kCRows, S.next_chunk);
-                S.cur_chunk = S.next_chunk;
-                S.cur_start += kCRows;
-                S.next_chunk = -1;
-            }
-            if (S.cur_chunk < 0) {
-                S.cur_chunk = atomicAdd(a.chunk_counter, 1);
-                a.item_first[item] = S.cur_chunk;
-            }
-            if (nrows + kTcBatch > S.cur_start + kCRows && S.next_chunk < 0)
-                S.next_chunk = atomicAdd(a.chunk_counter, 1);
+        return (s[0] + s[1]) + (s[2] + s[3]);
+    };
+    auto flush_direct = [&]() {
+        __syncwarp();
+        if (lane < nbuf * kVals) {
+            const int r = lane / kVals, c = lane - r * kVals;
+            const uint32_t g = s_gid[r];
+            const float s = lane_sum(lane);
+            atomicAdd(c == DD ? vden + g : vnum + (size_t)g * a.num_stride + c, s);
         }
-        const PairRec* rec = S.rec[slot];
-        const int cnt = (int)min((uint32_t)kTcBatch, range.y - (range.x + k * kTcBatch));
-        uint32_t lm = 0u;   // this lane's non-zero weights (bit j = Gaussian j)
-        if (__any_sync(0xffffffffu, !done)) {
-            // Gaussians of the batch that can reach this warp's pixel block,
-            // four at a time in list order: the four alphas are independent,
-            // the transmittance recursion then takes them in order
-            uint32_t rel = __ballot_sync(0xffffffffu, lane < cnt && ((rec[lane].mask >> warp) & 1u));
-            while (rel != 0u && __any_sync(0xffffffffu, !done)) {
-                int jj[4];
-                float al[4];
+        __syncwarp();
+        nbuf = 0;
+    };
+
+    for (uint32_t k = 0; k < nb && alive; ++k) {
+        const bool in = range.x + 32u * k + (uint32_t)lane < range.y;
+        const uint32_t gid = __float_as_uint(rb.z);
+        const uint32_t mask =
+            in ? (band_mask_fast(ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, tx, ty) >> band0) & ((1u << NB) - 1u) & alive : 0u;
+        __syncwarp();   // the previous batch's records have been read
+        s_rec[lane][0] = make_float4(ra.x, ra.x, ra.y, ra.y);
+        s_rec[lane][1] = make_float4(ra.z, ra.z, ra.w, ra.w);
+        s_rec[lane][2] = make_float4(rb.x, rb.x, rb.y, rb.y);
+        __syncwarp();
+        load_record(next_rank);
+        next_rank = rank_of(k + 2);
+        uint32_t B[NB], any = 0u;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    jj[q] = rel ? __ffs(rel) - 1 : -1;
-                    rel &= rel - 1u;
+        for (int b = 0; b < NB; ++b) {
+            B[b] = __ballot_sync(kAll, (mask >> b) & 1u);
+            any |= B[b];
+        }
+        uint32_t rowbits = 0u;
+        int myrow = -1;   // lane j: where entry j's row went
+#pragma unroll 1
+        for (int q = 0; q < 4 && any; ++q) {
+            uint32_t rel = any & (0xffu << (8 * q));
+            any &= ~rel;
+            while (rel) {
+                const int j = __ffs(rel) - 1;
+                const uint32_t bit = rel & (0u - rel);
+                rel ^= bit;
+                const ulonglong2 r0 = *reinterpret_cast<const ulonglong2*>(&s_rec[j][0]);
+                const ulonglong2 r1 = *reinterpret_cast<const ulonglong2*>(&s_rec[j][1]);
+                const ulonglong2 r2 = *reinterpret_cast<const ulonglong2*>(&s_rec[j][2]);
+                if (!kDirect && local == kCRows) {   // the next chunk
+                    int c = 0;
+                    if (lane == 0) {
+                        c = atomicAdd(a.chunk_counter, 1);
+                        if (cur < 0)
+                            a.item_first[item] = c;
+                        else
+                            finish_chunk(a, cur, kCRows, c);
+                    }
+                    cur = __shfl_sync(kAll, c, 0);
+                    local = 0;
+                    keep = cur < a.cap;
+                    d1 = a.wg1 + (size_t)cur * kChunkBytes + lane * 4;
+                    if (NT == 2) d2 = a.wg2 + (size_t)cur * kChunkBytes + lane * 4;
                 }
+                // the Gaussian's weights go to the next row's place as they are
+                // made; the place is taken only if one of them is not zero
+                const F2 dx = f2_add(F2{r0.x}, npx), adx2 = f2_mul(F2{r1.x}, f2_mul(dx, dx));
+                F2 acc[kDirect ? DD : 1], den = f2(0.f, 0.f);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int j = jj[q] < 0 ? jj[0] : jj[q];
-                    const float4 g = *reinterpret_cast<const float4*>(&rec[j].mx);
-                    const float2 h = *reinterpret_cast<const float2*>(&rec[j].cc);
-                    al[q] = alpha_at_nb(g.x, g.y, g.z, g.w, h.x, h.y, pxf, pyf);
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (jj[q] >= 0 && al[q] > 0.f && !done) {
-                        const float Tn = __fmul_rn(T, __fsub_rn(1.0f, al[q]));
-                        if (Tn < kTransMin) {
-                            done = true;
-                        } else {
-                            const float wv = __fmul_rn(al[q], T);
-                            T = Tn;
-                            lm |= 1u << jj[q];
-                            const int o = jj[q] * kRowBytes + pix * 2;
-                            const __nv_bfloat16 h1 = __float2bfloat16_rn(wv);
-                            *reinterpret_cast<__nv_bfloat16*>(&S.stage[0][o]) = h1;
-                            if (NT == 2)
-                                *reinterpret_cast<__nv_bfloat16*>(&S.stage[NT - 1][o]) =
-                                    __float2bfloat16_rn(wv - __bfloat162float(h1));
+                for (int c = 0; c < (kDirect ? DD : 1); ++c) acc[c] = f2(0.f, 0.f);
+                uint32_t nz = 0u;
+                auto band = [&](int b) {
+                    const float2 al = alpha_at_x2(dx, adx2, F2{r0.y}, F2{r1.y}, F2{r2.x}, F2{r2.y}, npy[b], one);
+                    // 1 - alpha, T (1 - alpha) and alpha T; a skipped pixel
+                    // (alpha 0) keeps its T, a pixel that would fall below
+                    // 1e-4 is done, one that is done stays so
+                    const F2 al2 = f2(al.x, al.y), t2 = f2(T[b][0], T[b][1]);
+                    const float2 tn = f2_get(f2_mul(t2, f2_fma(al2, f2(-1.f, -1.f), f2(1.f, 1.f))));
+                    const float2 ww = f2_get(f2_mul(al2, t2));
+                    T[b][0] = tn.x >= kTransMin ? tn.x : 0.f;
+                    T[b][1] = tn.y >= kTransMin ? tn.y : 0.f;
+                    const float wx = tn.x >= kTransMin ? ww.x : 0.f, wy = tn.y >= kTransMin ? ww.y : 0.f;
+                    nz |= __float_as_uint(wx) | __float_as_uint(wy);
+                    F2 wv = f2(wx, wy);
+                    if (!kDirect || NT == 1) {
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(wx, wy);
+                        const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
+                        const F2 hf = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u));
+                        if (!kDirect && keep) *reinterpret_cast<uint32_t*>(d1 + 128 * b) = hb;
+                        if (!kDirect && NT == 2) {   // w - h is exact
+                            const float2 res = f2_get(f2_fma(hf, f2(-1.f, -1.f), wv));
+                            const __nv_bfloat162 l = __floats2bfloat162_rn(res.x, res.y);
+                            const uint32_t lb = *reinterpret_cast<const uint32_t*>(&l);
+                            if (keep) *reinterpret_cast<uint32_t*>(d2 + 128 * b) = lb;
+                            if (!count)
+                                den = f2_add(den, f2(__uint_as_float(lb << 16), __uint_as_float(lb & 0xffff0000u)));
                         }
+                        wv = hf;
+                    }
+                    // den: the weights' sum, or the number of non-zero ones
+                    den = f2_add(den, count ? f2(wx > 0.f ? 1.f : 0.f, wy > 0.f ? 1.f : 0.f) : wv);
+                    if constexpr (kDirect) {
+#pragma unroll
+                        for (int c = 0; c < DD; ++c) acc[c] = f2_fma(wv, feat[c][b], acc[c]);
+                    }
+                };
+                auto band_or_zero = [&](int b) {
+                    if (B[b] & bit) {
+                        band(b);
+                    } else if (!kDirect && keep) {
+                        *reinterpret_cast<uint32_t*>(d1 + 128 * b) = 0u;
+                        if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + 128 * b) = 0u;
+                    }
+                };
+                // two bands at a time where both are reached (independent chains)
+#pragma unroll
+                for (int b = 0; b < NB; b += 2) {
+                    if (NB > 1 && (B[b] & B[NB > 1 ? b + 1 : b] & bit)) {
+                        band(b);
+                        band(NB > 1 ? b + 1 : b);
+                    } else {
+                        band_or_zero(b);
+                        if (NB > 1) band_or_zero(NB > 1 ? b + 1 : b);
                     }
                 }
+                if (!__any_sync(kAll, nz != 0u)) continue;
+                const float2 sd = f2_get(den);
+                if constexpr (kDirect) {
+                    float* p = s_part + nbuf * (kVals * 33) + lane;
+#pragma unroll
+                    for (int c = 0; c < DD; ++c) {
+                        const float2 s = f2_get(acc[c]);
+                        p[33 * c] = s.x + s.y;
+                    }
+                    p[33 * DD] = sd.x + sd.y;
+                    if (lane == j) s_gid[nbuf] = gid;
+                    if (++nbuf == kRowBuf) flush_direct();
+                } else {
+                    s_part[33 * nbuf + lane] = sd.x + sd.y;
+                    if (lane == j && keep) myrow = cur * kCRows + local;
+                    rowbits |= bit;
+                    ++nbuf;
+                    ++local;
+                    d1 += kRowBytes;
+                    if (NT == 2) d2 += kRowBytes;
+                }
             }
-            const uint32_t mine = __reduce_or_sync(0xffffffffu, lm);
-            if (lane == 0 && mine) atomicOr(&S.rowmask[buf], mine);
+            // bands whose pixels are all done take no further part
+            alive = 0u;
+            any = 0u;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                if (__any_sync(kAll, T[b][0] + T[b][1] > 0.f)) {
+                    alive |= 1u << b;
+                    any |= B[b];
+                } else {
+                    B[b] = 0u;
+                }
+            }
+            any &= q < 3 ? 0xffffffffu << (8 * q + 8) : 0u;
         }
-        if (warp == 0) mask_batch(k + 1);   // (pending: batches k+1 .. k+kRing-1)
-        if (tid == 0) S.rowmask[buf ^ 1] = 0u;
-        __syncthreads();
-        const uint32_t rowmask = S.rowmask[buf];
-        const int nnew = __popc(rowmask);
-        const int cur = S.cur_chunk, nxt = S.next_chunk, cstart = S.cur_start;
-        // the staging row of the i-th new Gaussian (the i-th set bit j of the
-        // row mask) goes to tile row nrows + i (chunk cur, or nxt past its 128
-        // rows), 16 bytes per lane, one warp per row and term; the staging row
-        // is cleared behind, the row's sum of each term (the bfloat16 values the
-        // product uses) is kept for den, and the Gaussian id is recorded
-        if constexpr (DIRECT) {
-            // warp i % 8 takes row i: its weights w = W1 (+ W2), 8 pixels per
-            // lane, dotted with the tile's channels; the staging row is cleared
-            float* const vnum = a.views.num[v];
-            float* const vden = a.views.den[v];
-            uint32_t m = rowmask;
-            for (int i = 0; m != 0u; ++i, m &= m - 1u) {
-                if ((i & 7) != warp) continue;
-                const int j = __ffs(m) - 1;
-                float w[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                float sden = 0.f;
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    uint4* src = reinterpret_cast<uint4*>(&S.stage[t][j * kRowBytes + lane * 16]);
-                    const uint4 v4 = *src;
-                    *src = make_uint4(0u, 0u, 0u, 0u);
-                    const uint32_t wv[4] = {v4.x, v4.y, v4.z, v4.w};
-                    sden += lane_den(wv, a.count_den, t);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        w[2 * k] += __uint_as_float(wv[k] << 16);
-                        w[2 * k + 1] += __uint_as_float(wv[k] & 0xffff0000u);
-                    }
-                }
-                sden = warp_sum(sden);   // the row's den over both terms
-                const uint32_t gid = rec[j].gid;
-#pragma unroll
-                for (int c = 0; c < kDirectMaxD; ++c) {
-                    if (c >= a.direct_d) break;
-                    const float4 f0 = *reinterpret_cast<const float4*>(&S.feat[c][lane * 8]);
-                    const float4 f1 = *reinterpret_cast<const float4*>(&S.feat[c][lane * 8 + 4]);
-                    float sc = w[0] * f0.x;
-                    sc = fmaf(w[1], f0.y, sc);
-                    sc = fmaf(w[2], f0.z, sc);
-                    sc = fmaf(w[3], f0.w, sc);
-                    sc = fmaf(w[4], f1.x, sc);
-                    sc = fmaf(w[5], f1.y, sc);
-                    sc = fmaf(w[6], f1.z, sc);
-                    sc = fmaf(w[7], f1.w, sc);
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-                    if (lane == 0) atomicAdd(vnum + (size_t)gid * a.num_stride + c, sc);
-                }
-                if (lane == 0) atomicAdd(vden + gid, sden);
+        if constexpr (!kDirect) {
+            // the rows' den and Gaussian, lane j for entry j's row
+            __syncwarp();
+            if (((rowbits >> lane) & 1u) && myrow >= 0) {
+                const float s = lane_sum(__popc(rowbits & lt_mask));
+                // the row's den in term 0's slot (the aggregation adds the slots)
+                a.chunk_den[(size_t)myrow * NT] = s;
+                if (NT == 2) a.chunk_den[(size_t)myrow * NT + 1] = 0.f;
+                a.chunk_gid[myrow] = gid;
             }
-        } else if constexpr (NT == 2) {
-            // warp i % 8 takes row i, both terms
-            uint32_t m = rowmask;
-            for (int i = 0; m != 0u; ++i, m &= m - 1u) {
-                if ((i & 7) != warp) continue;
-                const int j = __ffs(m) - 1;
-                int local = nrows + i - cstart, ch = cur;
-                if (local >= kCRows) {
-                    local -= kCRows;
-                    ch = nxt;
-                }
-                const bool keep = ch >= 0 && ch < a.cap;
-                float sden = 0.f;   // this lane's part of the row's den, both terms
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    uint4* src = reinterpret_cast<uint4*>(&S.stage[t][j * kRowBytes + lane * 16]);
-                    const uint4 v4 = *src;
-                    if (keep) {
-                        uint8_t* dst = (t == 0 ? a.wg1 : a.wg2) + (size_t)ch * kChunkBytes + local * kRowBytes + lane * 16;
-                        *reinterpret_cast<uint4*>(dst) = v4;
-                    }
-                    *src = make_uint4(0u, 0u, 0u, 0u);
-                    const uint32_t wv[4] = {v4.x, v4.y, v4.z, v4.w};
-                    sden += lane_den(wv, a.count_den, t);
-                }
-                sden = warp_sum(sden);
-                if (lane == 0 && keep) {
-                    // the row's den in term 0's slot (the aggregation adds the slots)
-                    a.chunk_den[((size_t)ch * kCRows + local) * NT] = sden;
-                    a.chunk_den[((size_t)ch * kCRows + local) * NT + 1] = 0.f;
-                    a.chunk_gid[(size_t)ch * kCRows + local] = rec[j].gid;
-                }
-            }
-        } else {
-            // warp w takes row w (row i of the 32 at most: warp i % 8 on pass i / 8)
-            for (int e = tid; e < nnew * 32; e += 256) {
-                const int i = e >> 5;
-                const int j = (int)__fns(rowmask, 0u, i + 1);
-                int local = nrows + i - cstart, ch = cur;
-                if (local >= kCRows) {
-                    local -= kCRows;
-                    ch = nxt;
-                }
-                uint4* src = reinterpret_cast<uint4*>(&S.stage[0][j * kRowBytes + lane * 16]);
-                const uint4 v4 = *src;
-                if (ch >= 0 && ch < a.cap)
-                    *reinterpret_cast<uint4*>(a.wg1 + (size_t)ch * kChunkBytes + local * kRowBytes + lane * 16) = v4;
-                *src = make_uint4(0u, 0u, 0u, 0u);
-                const uint32_t wv[4] = {v4.x, v4.y, v4.z, v4.w};
-                const float sden = row_den(wv, a.count_den, 0);
-                if (lane == 0 && ch >= 0 && ch < a.cap) a.chunk_den[(size_t)ch * kCRows + local] = sden;
-            }
-            if (tid < kTcBatch && ((rowmask >> tid) & 1u)) {
-                int local = nrows + __popc(rowmask & lt_mask) - cstart, ch = cur;
-                if (local >= kCRows) {
-                    local -= kCRows;
-                    ch = nxt;
-                }
-                if (ch >= 0 && ch < a.cap) a.chunk_gid[(size_t)ch * kCRows + local] = rec[tid].gid;
-            }
+            nbuf = 0;
         }
-        nrows += nnew;
-        // no barrier here: the next batch's counting barrier orders these stores
     }
-    // gathers issued past an early stop still land before the CTA exits
-    if (warp == 0) cp_async_wait<0>();
-    __syncthreads();
-    if (!DIRECT && tid == 0) {
-        const int cur = S.cur_chunk, cstart = S.cur_start, nxt = S.next_chunk;
-        if (nrows > cstart + kCRows) {   // the last batch spilled into nxt
-            finish_chunk(a, cur, kCRows, nxt);
-            finish_chunk(a, nxt, nrows - cstart - kCRows, -1);
-        } else {
-            finish_chunk(a, cur, nrows - cstart, -1);
-            finish_chunk(a, nxt, 0, -1);   // allocated, never used
-        }
+    if constexpr (kDirect) {
+        if (nbuf > 0) flush_direct();
+    } else {
+        if (lane == 0 && cur >= 0) finish_chunk(a, cur, local, -1);
     }
 }
 
@@ -1608,11 +1557,12 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         w.cap = (int)cap;
         w.chunk_den = t.cden;
         w.count_den = option_count_normalise() ? 1 : 0;
+        w.one = make_float2(1.f, 1.f);
         const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
         if (NT == 2)
-            k_weights<2, false><<<nitems, 256, 0, st>>>(w);
+            k_weights<2, 0, 4><<<nitems, 32, 0, st>>>(w);
         else
-            k_weights<1, false><<<nitems, 256, 0, st>>>(w);
+            k_weights<1, 0, 4><<<nitems, 32, 0, st>>>(w);
         LV_LAUNCH();
         trace_end(tslot, st);
         if (!checked) break;
@@ -1655,6 +1605,31 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
 // aggregation launch exist for the group.  The chunk counter stays 0.
 bool tc_direct_supported(int d) { return d >= 1 && d <= kDirectMaxD; }
 
+namespace {
+template <int NT, int NB>
+void launch_weights_direct_nb(const WeightsArgs& w, int d, int nitems, cudaStream_t st) {
+    const unsigned grid = (unsigned)nitems * (4 / NB);
+    switch (d) {
+        case 1: k_weights<NT, 1, NB><<<grid, 32, 0, st>>>(w); break;
+        case 2: k_weights<NT, 2, NB><<<grid, 32, 0, st>>>(w); break;
+        case 3: k_weights<NT, 3, NB><<<grid, 32, 0, st>>>(w); break;
+        default: k_weights<NT, 4, NB><<<grid, 32, 0, st>>>(w); break;
+    }
+}
+
+// Whole tiles per warp, or, when the tiles would not give every scheduler four
+// warps, one band per warp: a band's rows cost the lane sums of a whole row, but
+// the longest tile's chain is a quarter (8 views of 128x128, 512 tiles: 765 us a
+// call by tiles, 490 by bands; from 2432 tiles on the two are level).
+void launch_weights_direct(const WeightsArgs& w, int NT, int d, int nitems, cudaStream_t st) {
+    const bool bands = nitems < kBandItems;
+    if (NT == 2)
+        bands ? launch_weights_direct_nb<2, 1>(w, d, nitems, st) : launch_weights_direct_nb<2, 4>(w, d, nitems, st);
+    else
+        bands ? launch_weights_direct_nb<1, 1>(w, d, nitems, st) : launch_weights_direct_nb<1, 4>(w, d, nitems, st);
+}
+}  // namespace
+
 ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int height, int NT, int d, int num_stride,
                                 const void* feats, int feat_dtype, const AggViews& av, Arena& ws, int parity,
                                 int* status, bool checked, cudaStream_t st, int** counter) {
@@ -1679,16 +1654,12 @@ ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int heig
     w.height = height;
     w.chunk_counter = cnt;
     w.count_den = option_count_normalise() ? 1 : 0;
-    w.direct_d = d;
+    w.one = make_float2(1.f, 1.f);
     w.num_stride = num_stride;
     w.feats = feats;
-    w.feat_bf16 = feat_dtype == LUDVIG_BF16 ? 1 : 0;
     w.views = av;
     const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
-    if (NT == 2)
-        k_weights<2, true><<<nitems, 256, 0, st>>>(w);
-    else
-        k_weights<1, true><<<nitems, 256, 0, st>>>(w);
+    launch_weights_direct(w, NT, d, nitems, st);
     LV_LAUNCH();
     trace_end(tslot, st);
     if (checked) {
