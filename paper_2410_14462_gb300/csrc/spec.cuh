@@ -259,10 +259,11 @@ __device__ __forceinline__ F2 f2_sum(F2 a, F2 b, F2 one) { return f2_fma(a, one,
 // adding and subtracting 1.5 * 2^23 (round to nearest even, as rintf), and 2^n
 // goes into the exponent field by an integer add (exact where the result is
 // normal; elsewhere alpha is under 1/255 and skipped).
-// dx = mx - px and adx2 = ca (dx dx) are the caller's (the same for every row).
-__device__ __forceinline__ float2 alpha_at_x2(F2 dx, F2 adx2, F2 my, F2 cb, F2 cc, F2 op, F2 npy, F2 one) {
-    const F2 dy = f2_add(my, npy);
-    const F2 s = f2_sum(adx2, f2_mul(cc, f2_mul(dy, dy)), one);
+// The differences and their squares times the conic's diagonal, dx = mx - px
+// and ax = ca (dx dx), dy and cy likewise, are the caller's (pixels that share
+// a column or a row share them).
+__device__ __forceinline__ float2 alpha_at_x2(F2 dx, F2 ax, F2 dy, F2 cy, F2 cb, F2 op, F2 one) {
+    const F2 s = f2_sum(ax, cy, one);
     // (0.5 s is exact, so that product may be fused)
     const F2 m = f2_fma(f2(0.5f, 0.5f), s, f2_mul(cb, f2_mul(dx, dy)));
     constexpr float kRound = 12582912.0f;
@@ -282,10 +283,10 @@ __device__ __forceinline__ float2 alpha_at_x2(F2 dx, F2 adx2, F2 my, F2 cb, F2 c
     const float ex = __uint_as_float((__float_as_uint(tt.x) << 23) + __float_as_uint(pp.x));
     const float ey = __uint_as_float((__float_as_uint(tt.y) << 23) + __float_as_uint(pp.y));
     const float2 al = f2_get(f2_mul(op, f2(ex, ey)));
-    const float ax = fminf(al.x, kAlphaMax), ay = fminf(al.y, kAlphaMax);
+    const float a0 = fminf(al.x, kAlphaMax), a1 = fminf(al.y, kAlphaMax);
     const uint32_t lim = 0x42ae0000u;   // 87
-    return make_float2(__float_as_uint(mm.x) <= lim && ax >= kAlphaMin ? ax : 0.0f,
-                       __float_as_uint(mm.y) <= lim && ay >= kAlphaMin ? ay : 0.0f);
+    return make_float2(__float_as_uint(mm.x) <= lim && a0 >= kAlphaMin ? a0 : 0.0f,
+                       __float_as_uint(mm.y) <= lim && a1 >= kAlphaMin ? a1 : 0.0f);
 }
 
 // Conservative test: can a projected Gaussian reach alpha >= 1/255 at some
@@ -459,10 +460,10 @@ __device__ __forceinline__ uint32_t block_mask_fast(float mx, float my, float a,
     return m;
 }
 
-// The same test per 16x4 band of the tile (bit k: rows 4 k .. 4 k + 3), for
-// the weights pass, whose warps take a tile band by band.
-__device__ __forceinline__ uint32_t band_mask_fast(float mx, float my, float a, float b, float c, float op, int tx,
-                                                   int ty) {
+// The same test per 8x8 quadrant of the tile (bit w: offset ((w & 1) * 8,
+// (w >> 1) * 8)), for the weights pass, whose warps take a tile by quadrants.
+__device__ __forceinline__ uint32_t quadrant_mask_fast(float mx, float my, float a, float b, float c, float op, int tx,
+                                                       int ty) {
     if (op < kAlphaMin) return 0u;
     const float thr = 2.0f * __logf(255.0f * op) * 1.001f + 1e-3f;
     const float det = a * c - b * b;
@@ -476,14 +477,16 @@ __device__ __forceinline__ uint32_t band_mask_fast(float mx, float my, float a, 
     const float xt = (float)(tx * kTile) + 0.5f, yt = (float)(ty * kTile) + 0.5f;
     uint32_t m = 0u;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float ylo = yt + (float)(4 * k);
-        const float w0 = fmaxf(my - (ylo + 3.0f), -wmax), w1 = fminf(my - ylo, wmax);
+    for (int k = 0; k < 2; ++k) {
+        const float ylo = yt + (float)(8 * k);
+        const float w0 = fmaxf(my - (ylo + 7.0f), -wmax), w1 = fminf(my - ylo, wmax);
         if (w0 > w1) continue;
         const float s0 = sqrt_approx(thra - det * w0 * w0), s1 = sqrt_approx(thra - det * w1 * w1);
         const float hi = (ws >= w0 && ws <= w1) ? umax : fmaxf((-b * w0 + s0) * inv_a, (-b * w1 + s1) * inv_a);
         const float lo = (-ws >= w0 && -ws <= w1) ? -umax : fminf((-b * w0 - s0) * inv_a, (-b * w1 - s1) * inv_a);
-        if (mx - lo + epsx >= xt && mx - hi - epsx <= xt + 15.0f) m |= 1u << k;
+        const float xl = mx - hi - epsx, xr = mx - lo + epsx;
+        if (xr >= xt && xl <= xt + 7.0f) m |= 1u << (2 * k);
+        if (xr >= xt + 8.0f && xl <= xt + 15.0f) m |= 1u << (2 * k + 1);
     }
     return m;
 }

@@ -98,7 +98,6 @@ struct WeightsArgs {
     int cap;
     float* chunk_den;       // [cap][128][NT]: each row's den, the sum of its weight terms, in term 0's
                             // slot (term 1's: 0); rewritten on a re-run
-    int count_den;          // chunk_den holds each row's count of non-zero weights instead
     // direct accumulation (k_weights<NT, true>, few channels): each new row's
     // sum_p w F[p, c] and its den go straight into the view's num and den
     // (atomic adds); no weight rows, chunks or plan are written
@@ -109,7 +108,7 @@ struct WeightsArgs {
 };
 
 constexpr int kDirectMaxD = 4;
-constexpr int kBandItems = 152 * 16;
+constexpr int kQuadItems = 152 * 16;
 
 __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int rows, int next) {
     if (c >= 0 && c < a.cap) {
@@ -118,34 +117,37 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
     }
 }
 
-// The weights of one (view, tile), a warp per tile (NB = 4) or per 16x4 band of
-// it (NB = 1): band b is the tile's pixels 64 b .. 64 b + 63, lane l holds
-// pixels 64 b + 2 l and + 1.
+// The weights of one (view, tile), a warp per tile (NB = 4) or per 8x8 quadrant
+// of it (NB = 1); a lane holds two neighbouring pixels of each quadrant.
 //   DD = 0: weight rows; DD = 1 .. 4: direct accumulation of DD channels.
+//   COUNT: den is the number of a row's non-zero weights instead of their sum.
 //
-// Bound: instruction issue (half FMA pipe, half ALU), with the launch's tail
-// (0.25 to 0.4 ms until the longest tiles end) next to it; a paper-scale tile
-// walks about 210 of its 2200 entries, 550 (entry, band) pairs.  Hence
+// Bound: instruction issue (0.74 of it, FMA pipe and ALU half busy each), with
+// the launch's tail (0.2 to 0.4 ms until the longest tiles end) next to it; a
+// paper-scale tile walks about 210 of its 2200 entries, 490 (entry, quadrant)
+// pairs.  Hence
 //  - two pixels per lane: Blackwell's packed float32 instructions halve the
-//    arithmetic's issue slots (25 packed operations per 64 pixels);
+//    arithmetic's issue slots (about 20 packed operations per 64 pixels, the
+//    column's and the row's terms shared between quadrants);
 //  - a warp owns the tile, so nothing waits at a block barrier and a row of
-//    256 pixels leaves as one coalesced 128-byte store per band and term,
-//    without staging; entries are skipped per band (a bit mask per entry);
+//    256 pixels is stored from registers, without staging;
+//  - entries are skipped per quadrant (a bit mask per entry); 16x4 bands, whose
+//    row stores are contiguous, evaluate 11 to 18 % more pairs and took 12 to
+//    14 % longer;
 //  - a row's lane sums wait in shared memory and are added up with one lane per
 //    row (2 instructions a row where a shuffle reduction takes 10), and so are
-//    the few channels of the direct form, whose atomics then come 32 at once;
-//  - where both bands of a pair are reached they are computed side by side, for
-//    the long tiles that end a launch.
-// 28 warps per SM (72 registers): 20, 24 and 32 measured 2.95, 2.78 and 2.65 ms
-// against 2.62.  20 paper-scale views (1M Gaussians, 980x546, float32): 4.30 ->
-// 2.62 ms against one block of 8 warps per tile with a weight row staged in
-// shared memory; 48 views of 640x480, bfloat16 rows: 6.40 -> 4.0 ms; 60 views
-// of 640x480, 3 channels direct: 6.81 -> 3.75 ms.
-template <int NT, int DD, int NB>
+//    the few channels of the direct form, whose atomics then come 32 at once.
+// 28 warps per SM (72 registers); 20, 24 and 32 were 10, 5 and 0 % slower.
+// 20 paper-scale views (1M Gaussians, 980x546, float32): 4.30 -> 2.22 ms against
+// one block of 8 warps per tile that staged a batch's rows in shared memory; 48
+// views of 640x480, bfloat16 rows: 6.40 -> 3.37 ms; 60 views of 640x480, 3
+// channels direct: 6.81 -> 3.3 ms.
+template <int NT, int DD, int NB, bool COUNT>
 __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_constant__ WeightsArgs a) {
     constexpr bool kDirect = DD > 0;
     constexpr int kVals = kDirect ? DD + 1 : 1;   // sums per row
     constexpr int kRowBuf = 32 / kVals;           // rows whose lane sums are kept
+    constexpr int kGroup = NB == 1 ? 2 : 1;       // entries taken together
     constexpr uint32_t kAll = 0xffffffffu;
     __shared__ float4 s_rec[32][3];               // the batch's records, every value twice
     __shared__ float s_part[32 * 33];             // [row][sum][lane]
@@ -153,29 +155,34 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
     const int lane = threadIdx.x;
     const uint32_t lt_mask = (1u << lane) - 1u;
     const int item = NB == 4 ? (int)blockIdx.x : (int)(blockIdx.x >> 2);
-    const int band0 = NB == 4 ? 0 : (int)(blockIdx.x & 3u);
+    const int quad0 = NB == 4 ? 0 : (int)(blockIdx.x & 3u);
     const uint2 range = a.ranges[item];
     if (range.x >= range.y) return;
     const int v = item / a.ntiles, tile = item - v * a.ntiles;
     const int tx = tile % a.TX, ty = tile / a.TX;
-    const int px = tx * kTile + 2 * (lane & 7), py = ty * kTile + 4 * band0 + (lane >> 3);
-    const F2 npx = f2(-((float)px + 0.5f), -((float)px + 1.5f));
+    // quadrant q's pixels of this lane: (px + 8 (q & 1), + 1; py + 8 (q >> 1))
+    constexpr int kCols = NB == 4 ? 2 : 1;
+    const int px = tx * kTile + 8 * (quad0 & 1) + 2 * (lane & 3), py = ty * kTile + 8 * (quad0 >> 1) + (lane >> 2);
     const F2 one = f2(a.one.x, a.one.y);
-    const bool count = a.count_den != 0;
-    F2 npy[NB];
+    F2 npx[kCols], npy[kCols];
     float T[NB][2];   // transmittance; 0 once the pixel is done
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const float y = -((float)(py + 4 * b) + 0.5f);
-        npy[b] = f2(y, y);
-        T[b][0] = px < a.width && py + 4 * b < a.height ? 1.0f : 0.0f;
-        T[b][1] = px + 1 < a.width && py + 4 * b < a.height ? 1.0f : 0.0f;
+    for (int h = 0; h < kCols; ++h) {
+        const float x = (float)(px + 8 * h), y = -((float)(py + 8 * h) + 0.5f);
+        npx[h] = f2(-(x + 0.5f), -(x + 1.5f));
+        npy[h] = f2(y, y);
     }
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            T[b][q] = px + 8 * (b & 1) + q < a.width && py + 8 * (b >> 1) < a.height ? 1.0f : 0.0f;
     F2 feat[kDirect ? DD : 1][NB];
     if constexpr (kDirect) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-            const size_t p = ((size_t)a.views.fview[v] * a.height + (py + 4 * b)) * a.width + px;
+            const size_t p =
+                ((size_t)a.views.fview[v] * a.height + (py + 8 * (b >> 1))) * a.width + (px + 8 * (b & 1));
 #pragma unroll
             for (int c = 0; c < DD; ++c) {
                 float x[2] = {0.f, 0.f};
@@ -206,18 +213,19 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
     load_record(rank_of(0));
     uint32_t next_rank = rank_of(1);
 
-    uint32_t alive = 0u;   // bands with a pixel that is not done
+    uint32_t alive = 0u;   // quadrants with a pixel that is not done
 #pragma unroll
     for (int b = 0; b < NB; ++b) alive |= __any_sync(kAll, T[b][0] + T[b][1] > 0.f) ? 1u << b : 0u;
 
     int cur = -1, local = kCRows;   // the tile's chunk being filled and its rows so far
-    bool keep = false;
     uint8_t *d1 = nullptr, *d2 = nullptr;
     int nbuf = 0;   // rows in s_part
     const uint32_t nb = (range.y - range.x + 31u) / 32u;
     float* const vnum = kDirect ? a.views.num[v] : nullptr;
     float* const vden = kDirect ? a.views.den[v] : nullptr;
     // sum `i` of the kept rows over the lanes
+    // byte of quadrant b's first pixel in a row
+    auto kQuadByte = [](int b) { return (b >> 1) * 256 + (b & 1) * 16; };
     auto lane_sum = [&](int i) {
         const float* p = s_part + 33 * i;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -246,7 +254,7 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
         const bool in = range.x + 32u * k + (uint32_t)lane < range.y;
         const uint32_t gid = __float_as_uint(rb.z);
         const uint32_t mask =
-            in ? (band_mask_fast(ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, tx, ty) >> band0) & ((1u << NB) - 1u) & alive : 0u;
+            in ? (quadrant_mask_fast(ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, tx, ty) >> quad0) & ((1u << NB) - 1u) & alive : 0u;
         __syncwarp();   // the previous batch's records have been read
         s_rec[lane][0] = make_float4(ra.x, ra.x, ra.y, ra.y);
         s_rec[lane][1] = make_float4(ra.z, ra.z, ra.w, ra.w);
@@ -267,12 +275,33 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
             uint32_t rel = any & (0xffu << (8 * q));
             any &= ~rel;
             while (rel) {
-                const int j = __ffs(rel) - 1;
-                const uint32_t bit = rel & (0u - rel);
-                rel ^= bit;
-                const ulonglong2 r0 = *reinterpret_cast<const ulonglong2*>(&s_rec[j][0]);
-                const ulonglong2 r1 = *reinterpret_cast<const ulonglong2*>(&s_rec[j][1]);
-                const ulonglong2 r2 = *reinterpret_cast<const ulonglong2*>(&s_rec[j][2]);
+                // kGroup entries at a time: their alphas are independent, the
+                // transmittances take them in order
+                F2 dx[kGroup][kCols], ax[kGroup][kCols], dy[kGroup][kCols], cy[kGroup][kCols], cb[kGroup], op[kGroup];
+                int je[kGroup];
+                uint32_t bits[kGroup];
+#pragma unroll
+                for (int g = 0; g < kGroup; ++g) {
+                    bits[g] = rel & (0u - rel);
+                    rel ^= bits[g];
+                    je[g] = g == 0 || bits[g] ? __ffs(bits[g]) - 1 : je[0];
+                    const ulonglong2 r0 = *reinterpret_cast<const ulonglong2*>(&s_rec[je[g]][0]);
+                    const ulonglong2 r1 = *reinterpret_cast<const ulonglong2*>(&s_rec[je[g]][1]);
+                    const ulonglong2 r2 = *reinterpret_cast<const ulonglong2*>(&s_rec[je[g]][2]);
+#pragma unroll
+                    for (int h = 0; h < kCols; ++h) {
+                        dx[g][h] = f2_add(F2{r0.x}, npx[h]);
+                        ax[g][h] = f2_mul(F2{r1.x}, f2_mul(dx[g][h], dx[g][h]));
+                        dy[g][h] = f2_add(F2{r0.y}, npy[h]);
+                        cy[g][h] = f2_mul(F2{r2.x}, f2_mul(dy[g][h], dy[g][h]));
+                    }
+                    cb[g] = F2{r1.y};
+                    op[g] = F2{r2.y};
+                }
+                auto alpha = [&](int g, int b) {
+                    const int h = b & 1, k = NB == 4 ? b >> 1 : 0;
+                    return alpha_at_x2(dx[g][h], ax[g][h], dy[g][k], cy[g][k], cb[g], op[g], one);
+                };
                 if (!kDirect && local == kCRows) {   // the next chunk
                     int c = 0;
                     if (lane == 0) {
@@ -284,94 +313,109 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                     }
                     cur = __shfl_sync(kAll, c, 0);
                     local = 0;
-                    keep = cur < a.cap;
-                    d1 = a.wg1 + (size_t)cur * kChunkBytes + lane * 4;
-                    if (NT == 2) d2 = a.wg2 + (size_t)cur * kChunkBytes + lane * 4;
+                    // (a launch that runs out of chunks is redone: what it
+                    // writes to the last one is not used)
+                    const size_t o = (size_t)min(cur, a.cap - 1) * kChunkBytes + (lane >> 2) * 32 + (lane & 3) * 4;
+                    d1 = a.wg1 + o;
+                    if (NT == 2) d2 = a.wg2 + o;
                 }
-                // the Gaussian's weights go to the next row's place as they are
-                // made; the place is taken only if one of them is not zero
-                const F2 dx = f2_add(F2{r0.x}, npx), adx2 = f2_mul(F2{r1.x}, f2_mul(dx, dx));
-                F2 acc[kDirect ? DD : 1], den = f2(0.f, 0.f);
+                float2 al1[kGroup];   // NB = 1: the group's alphas
+                if constexpr (NB == 1) {
 #pragma unroll
-                for (int c = 0; c < (kDirect ? DD : 1); ++c) acc[c] = f2(0.f, 0.f);
-                uint32_t nz = 0u;
-                auto band = [&](int b) {
-                    const float2 al = alpha_at_x2(dx, adx2, F2{r0.y}, F2{r1.y}, F2{r2.x}, F2{r2.y}, npy[b], one);
-                    // 1 - alpha, T (1 - alpha) and alpha T; a skipped pixel
-                    // (alpha 0) keeps its T, a pixel that would fall below
-                    // 1e-4 is done, one that is done stays so
-                    const F2 al2 = f2(al.x, al.y), t2 = f2(T[b][0], T[b][1]);
-                    const float2 tn = f2_get(f2_mul(t2, f2_fma(al2, f2(-1.f, -1.f), f2(1.f, 1.f))));
-                    const float2 ww = f2_get(f2_mul(al2, t2));
-                    T[b][0] = tn.x >= kTransMin ? tn.x : 0.f;
-                    T[b][1] = tn.y >= kTransMin ? tn.y : 0.f;
-                    const float wx = tn.x >= kTransMin ? ww.x : 0.f, wy = tn.y >= kTransMin ? ww.y : 0.f;
-                    nz |= __float_as_uint(wx) | __float_as_uint(wy);
-                    F2 wv = f2(wx, wy);
-                    if (!kDirect || NT == 1) {
-                        const __nv_bfloat162 h = __floats2bfloat162_rn(wx, wy);
-                        const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
-                        const F2 hf = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u));
-                        if (!kDirect && keep) *reinterpret_cast<uint32_t*>(d1 + 128 * b) = hb;
-                        if (!kDirect && NT == 2) {   // w - h is exact
-                            const float2 res = f2_get(f2_fma(hf, f2(-1.f, -1.f), wv));
-                            const __nv_bfloat162 l = __floats2bfloat162_rn(res.x, res.y);
-                            const uint32_t lb = *reinterpret_cast<const uint32_t*>(&l);
-                            if (keep) *reinterpret_cast<uint32_t*>(d2 + 128 * b) = lb;
-                            if (!count)
-                                den = f2_add(den, f2(__uint_as_float(lb << 16), __uint_as_float(lb & 0xffff0000u)));
+                    for (int g = 0; g < kGroup; ++g) al1[g] = alpha(g, 0);
+                }
+#pragma unroll
+                for (int g = 0; g < kGroup; ++g) {
+                    const int j = je[g];
+                    const uint32_t bit = bits[g];
+                    if (g > 0 && bit == 0u) continue;
+                    // the Gaussian's weights go to the next row's place as they
+                    // are made; the place is taken only if one of them is not zero
+                    F2 acc[kDirect ? DD : 1], den = f2(0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < (kDirect ? DD : 1); ++c) acc[c] = f2(0.f, 0.f);
+                    uint32_t nz = 0u;
+                    auto finish = [&](int b, float2 al) {
+                        // 1 - alpha, T (1 - alpha) and alpha T; a skipped pixel
+                        // (alpha 0) keeps its T, a pixel that would fall below
+                        // 1e-4 is done, one that is done stays so
+                        const F2 al2 = f2(al.x, al.y), t2 = f2(T[b][0], T[b][1]);
+                        const float2 tn = f2_get(f2_mul(t2, f2_fma(al2, f2(-1.f, -1.f), f2(1.f, 1.f))));
+                        const float2 ww = f2_get(f2_mul(al2, t2));
+                        T[b][0] = tn.x >= kTransMin ? tn.x : 0.f;
+                        T[b][1] = tn.y >= kTransMin ? tn.y : 0.f;
+                        const float wx = tn.x >= kTransMin ? ww.x : 0.f, wy = tn.y >= kTransMin ? ww.y : 0.f;
+                        nz |= __float_as_uint(wx) | __float_as_uint(wy);
+                        F2 wv = f2(wx, wy);
+                        if (!kDirect || NT == 1) {
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(wx, wy);
+                            const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
+                            const F2 hf = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u));
+                            if (!kDirect) *reinterpret_cast<uint32_t*>(d1 + kQuadByte(b)) = hb;
+                            if (!kDirect && NT == 2) {   // w - h is exact
+                                const float2 res = f2_get(f2_fma(hf, f2(-1.f, -1.f), wv));
+                                const __nv_bfloat162 l = __floats2bfloat162_rn(res.x, res.y);
+                                const uint32_t lb = *reinterpret_cast<const uint32_t*>(&l);
+                                *reinterpret_cast<uint32_t*>(d2 + kQuadByte(b)) = lb;
+                                if (!COUNT)
+                                    den = f2_add(den, f2(__uint_as_float(lb << 16), __uint_as_float(lb & 0xffff0000u)));
+                            }
+                            wv = hf;
                         }
-                        wv = hf;
-                    }
-                    // den: the weights' sum, or the number of non-zero ones
-                    den = f2_add(den, count ? f2(wx > 0.f ? 1.f : 0.f, wy > 0.f ? 1.f : 0.f) : wv);
-                    if constexpr (kDirect) {
+                        // den: the weights' sum, or the number of non-zero ones
+                        den = f2_add(den, COUNT ? f2(wx > 0.f ? 1.f : 0.f, wy > 0.f ? 1.f : 0.f) : wv);
+                        if constexpr (kDirect) {
 #pragma unroll
-                        for (int c = 0; c < DD; ++c) acc[c] = f2_fma(wv, feat[c][b], acc[c]);
-                    }
-                };
-                auto band_or_zero = [&](int b) {
-                    if (B[b] & bit) {
-                        band(b);
-                    } else if (!kDirect && keep) {
-                        *reinterpret_cast<uint32_t*>(d1 + 128 * b) = 0u;
-                        if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + 128 * b) = 0u;
-                    }
-                };
-                // two bands at a time where both are reached (independent chains)
-#pragma unroll
-                for (int b = 0; b < NB; b += 2) {
-                    if (NB > 1 && (B[b] & B[NB > 1 ? b + 1 : b] & bit)) {
-                        band(b);
-                        band(NB > 1 ? b + 1 : b);
+                            for (int c = 0; c < DD; ++c) acc[c] = f2_fma(wv, feat[c][b], acc[c]);
+                        }
+                    };
+                    if constexpr (NB == 1) {
+                        finish(0, al1[g]);
                     } else {
-                        band_or_zero(b);
-                        if (NB > 1) band_or_zero(NB > 1 ? b + 1 : b);
-                    }
-                }
-                if (!__any_sync(kAll, nz != 0u)) continue;
-                const float2 sd = f2_get(den);
-                if constexpr (kDirect) {
-                    float* p = s_part + nbuf * (kVals * 33) + lane;
+                        auto quad_or_zero = [&](int b) {
+                            if (B[b] & bit) {
+                                finish(b, alpha(g, b));
+                            } else if (!kDirect) {
+                                *reinterpret_cast<uint32_t*>(d1 + kQuadByte(b)) = 0u;
+                                if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + kQuadByte(b)) = 0u;
+                            }
+                        };
+                        // side by side where all four are reached (independent chains)
+                        if (B[0] & B[1] & B[2] & B[3] & bit) {
+                            float2 al[NB];
 #pragma unroll
-                    for (int c = 0; c < DD; ++c) {
-                        const float2 s = f2_get(acc[c]);
-                        p[33 * c] = s.x + s.y;
+                            for (int b = 0; b < NB; ++b) al[b] = alpha(g, b);
+#pragma unroll
+                            for (int b = 0; b < NB; ++b) finish(b, al[b]);
+                        } else {
+#pragma unroll
+                            for (int b = 0; b < NB; ++b) quad_or_zero(b);
+                        }
                     }
-                    p[33 * DD] = sd.x + sd.y;
-                    if (lane == j) s_gid[nbuf] = gid;
-                    if (++nbuf == kRowBuf) flush_direct();
-                } else {
-                    s_part[33 * nbuf + lane] = sd.x + sd.y;
-                    if (lane == j && keep) myrow = cur * kCRows + local;
-                    rowbits |= bit;
-                    ++nbuf;
-                    ++local;
-                    d1 += kRowBytes;
-                    if (NT == 2) d2 += kRowBytes;
+                    if (!__any_sync(kAll, nz != 0u)) continue;
+                    const float2 sd = f2_get(den);
+                    if constexpr (kDirect) {
+                        float* p = s_part + nbuf * (kVals * 33) + lane;
+#pragma unroll
+                        for (int c = 0; c < DD; ++c) {
+                            const float2 s = f2_get(acc[c]);
+                            p[33 * c] = s.x + s.y;
+                        }
+                        p[33 * DD] = sd.x + sd.y;
+                        if (lane == j) s_gid[nbuf] = gid;
+                        if (++nbuf == kRowBuf) flush_direct();
+                    } else {
+                        s_part[33 * nbuf + lane] = sd.x + sd.y;
+                        if (lane == j && cur < a.cap) myrow = cur * kCRows + local;
+                        rowbits |= bit;
+                        ++nbuf;
+                        ++local;
+                        d1 += kRowBytes;
+                        if (NT == 2) d2 += kRowBytes;
+                    }
                 }
             }
-            // bands whose pixels are all done take no further part
+            // quadrants whose pixels are all done take no further part
             alive = 0u;
             any = 0u;
 #pragma unroll
@@ -1556,13 +1600,13 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         w.chunk_counter = t.counter;
         w.cap = (int)cap;
         w.chunk_den = t.cden;
-        w.count_den = option_count_normalise() ? 1 : 0;
         w.one = make_float2(1.f, 1.f);
         const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
+        const bool count = option_count_normalise();
         if (NT == 2)
-            k_weights<2, 0, 4><<<nitems, 32, 0, st>>>(w);
+            count ? k_weights<2, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<2, 0, 4, false><<<nitems, 32, 0, st>>>(w);
         else
-            k_weights<1, 0, 4><<<nitems, 32, 0, st>>>(w);
+            count ? k_weights<1, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<1, 0, 4, false><<<nitems, 32, 0, st>>>(w);
         LV_LAUNCH();
         trace_end(tslot, st);
         if (!checked) break;
@@ -1606,27 +1650,28 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
 bool tc_direct_supported(int d) { return d >= 1 && d <= kDirectMaxD; }
 
 namespace {
-template <int NT, int NB>
+template <int NT, int NB, bool COUNT>
 void launch_weights_direct_nb(const WeightsArgs& w, int d, int nitems, cudaStream_t st) {
     const unsigned grid = (unsigned)nitems * (4 / NB);
     switch (d) {
-        case 1: k_weights<NT, 1, NB><<<grid, 32, 0, st>>>(w); break;
-        case 2: k_weights<NT, 2, NB><<<grid, 32, 0, st>>>(w); break;
-        case 3: k_weights<NT, 3, NB><<<grid, 32, 0, st>>>(w); break;
-        default: k_weights<NT, 4, NB><<<grid, 32, 0, st>>>(w); break;
+        case 1: k_weights<NT, 1, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
+        case 2: k_weights<NT, 2, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
+        case 3: k_weights<NT, 3, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
+        default: k_weights<NT, 4, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
     }
 }
 
-// Whole tiles per warp, or, when the tiles would not give every scheduler four
-// warps, one band per warp: a band's rows cost the lane sums of a whole row, but
-// the longest tile's chain is a quarter (8 views of 128x128, 512 tiles: 765 us a
-// call by tiles, 490 by bands; from 2432 tiles on the two are level).
-void launch_weights_direct(const WeightsArgs& w, int NT, int d, int nitems, cudaStream_t st) {
-    const bool bands = nitems < kBandItems;
-    if (NT == 2)
-        bands ? launch_weights_direct_nb<2, 1>(w, d, nitems, st) : launch_weights_direct_nb<2, 4>(w, d, nitems, st);
+template <int NT>
+void launch_weights_direct(const WeightsArgs& w, int d, int nitems, cudaStream_t st) {
+    // Whole tiles per warp, or, when the tiles would not give every scheduler
+    // four warps, one quadrant per warp: a quadrant's rows cost the lane sums of
+    // a whole row, but the longest tile's chain is a quarter (8 views of 128x128,
+    // 512 tiles: 470 us by tiles, 182 by quadrants; 2048 tiles: 590 and 400)
+    const bool quads = nitems < kQuadItems;
+    if (option_count_normalise())
+        quads ? launch_weights_direct_nb<NT, 1, true>(w, d, nitems, st) : launch_weights_direct_nb<NT, 4, true>(w, d, nitems, st);
     else
-        bands ? launch_weights_direct_nb<1, 1>(w, d, nitems, st) : launch_weights_direct_nb<1, 4>(w, d, nitems, st);
+        quads ? launch_weights_direct_nb<NT, 1, false>(w, d, nitems, st) : launch_weights_direct_nb<NT, 4, false>(w, d, nitems, st);
 }
 }  // namespace
 
@@ -1653,13 +1698,15 @@ ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int heig
     w.width = width;
     w.height = height;
     w.chunk_counter = cnt;
-    w.count_den = option_count_normalise() ? 1 : 0;
     w.one = make_float2(1.f, 1.f);
     w.num_stride = num_stride;
     w.feats = feats;
     w.views = av;
     const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
-    launch_weights_direct(w, NT, d, nitems, st);
+    if (NT == 2)
+        launch_weights_direct<2>(w, d, nitems, st);
+    else
+        launch_weights_direct<1>(w, d, nitems, st);
     LV_LAUNCH();
     trace_end(tslot, st);
     if (checked) {
