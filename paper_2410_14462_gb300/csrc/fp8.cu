@@ -9,7 +9,7 @@
 // Three passes over the features: a per-view maximum of |x| (the float bits
 // of non-negative values order like unsigned integers, so atomicMax on them
 // is exact), the scales, and the rounding of x / s_v (IEEE division, then the
-// hardware's round-to-nearest-even E4M3 conversion), four values per thread.
+// hardware's round-to-nearest-even E4M3 conversion).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -19,18 +19,65 @@ namespace ludvig {
 
 namespace {
 
+// Both passes take a view's elements in pieces of kPieces x 256 groups of four
+// (float32) or eight (bfloat16): 16-byte loads, kPieces of them in flight per
+// thread.  A view that does not start on a 16-byte boundary (or whose codes do
+// not start on one of a group's size), and the end of a view, go element by
+// element.
+constexpr int kPieces = 4;
+
+template <class T>
+struct Vec {
+    static constexpr int kN = 16 / (int)sizeof(T);
+    float x[kN];
+};
+__device__ __forceinline__ void load_vec(const float* p, Vec<float>& v) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v.x[0] = q.x;
+    v.x[1] = q.y;
+    v.x[2] = q.z;
+    v.x[3] = q.w;
+}
+__device__ __forceinline__ void load_vec(const __nv_bfloat16* p, Vec<__nv_bfloat16>& v) {
+    const uint4 q = *reinterpret_cast<const uint4*>(p);
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v.x[2 * k] = __uint_as_float(w[k] << 16);
+        v.x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+    }
+}
 __device__ __forceinline__ float load_x(const float* p, int64_t i) { return p[i]; }
 __device__ __forceinline__ float load_x(const __nv_bfloat16* p, int64_t i) { return __bfloat162float(p[i]); }
 
-// blockIdx.y = view; grid-stride over the view's elements.
+template <class T>
+constexpr int64_t piece_elems() {
+    return (int64_t)kPieces * 256 * Vec<T>::kN;
+}
+
+// blockIdx.y = view; grid-stride over the view's pieces.
 template <class T>
 __global__ void __launch_bounds__(256) k_view_absmax(const T* __restrict__ x, int64_t view_elems,
                                                      uint32_t* __restrict__ amax_bits) {
+    constexpr int kN = Vec<T>::kN;
     const T* xv = x + (int64_t)blockIdx.y * view_elems;
+    const bool vec = (reinterpret_cast<uintptr_t>(xv) & 15) == 0;
     float m = 0.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < view_elems;
-         i += (int64_t)gridDim.x * blockDim.x)
-        m = fmaxf(m, fabsf(load_x(xv, i)));
+    for (int64_t e0 = (int64_t)blockIdx.x * piece_elems<T>(); e0 < view_elems;
+         e0 += (int64_t)gridDim.x * piece_elems<T>()) {
+        if (vec && e0 + piece_elems<T>() <= view_elems) {
+            Vec<T> v[kPieces];
+#pragma unroll
+            for (int k = 0; k < kPieces; ++k) load_vec(xv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN, v[k]);
+#pragma unroll
+            for (int k = 0; k < kPieces; ++k)
+#pragma unroll
+                for (int q = 0; q < kN; ++q) m = fmaxf(m, fabsf(v[k].x[q]));
+        } else {
+            const int64_t e1 = min(view_elems, e0 + piece_elems<T>());
+            for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) m = fmaxf(m, fabsf(load_x(xv, e)));
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     __shared__ float wm[8];
@@ -55,20 +102,40 @@ __device__ __forceinline__ uint32_t e4m3_of(float x, float s) {
     return (uint32_t)__nv_cvt_float_to_fp8(__fdiv_rn(x, s), __NV_SATFINITE, __NV_E4M3);
 }
 
-// Thread t rounds elements 4t .. 4t + 3 of the whole array (one 4-byte store;
-// the scalar tail covers a total that is not a multiple of 4).
+// blockIdx.y = view, blockIdx.x = piece of it.  Bound by HBM (5 or 3 bytes per
+// element): 12 float32 views of 640x480x512 in 1.26 ms = 7.5 TB/s (3.14 ms with a
+// 64-bit division and a 4-byte load per element); the maximum 1.24 -> 1.05 ms.
 template <class T>
-__global__ void k_quantize_e4m3(const T* __restrict__ x, const float* __restrict__ s, int64_t view_elems,
-                                int64_t total, uint8_t* __restrict__ q) {
-    const int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (e0 >= total) return;
-    if (e0 + 4 <= total) {
-        uint32_t w = 0;
+__global__ void __launch_bounds__(256) k_quantize_e4m3(const T* __restrict__ x, const float* __restrict__ scales,
+                                                       int64_t view_elems, uint8_t* __restrict__ q) {
+    constexpr int kN = Vec<T>::kN;
+    const T* xv = x + (int64_t)blockIdx.y * view_elems;
+    uint8_t* qv = q + (int64_t)blockIdx.y * view_elems;
+    const float s = scales[blockIdx.y];
+    const int64_t e0 = (int64_t)blockIdx.x * piece_elems<T>();
+    const bool vec = ((reinterpret_cast<uintptr_t>(xv) & 15) | (reinterpret_cast<uintptr_t>(qv) & (kN - 1))) == 0;
+    if (vec && e0 + piece_elems<T>() <= view_elems) {
+        Vec<T> v[kPieces];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) w |= e4m3_of(load_x(x, e0 + k), s[(e0 + k) / view_elems]) << (8 * k);
-        *reinterpret_cast<uint32_t*>(q + e0) = w;
+        for (int k = 0; k < kPieces; ++k) load_vec(xv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN, v[k]);
+#pragma unroll
+        for (int k = 0; k < kPieces; ++k) {
+            uint32_t w[kN / 4];
+#pragma unroll
+            for (int h = 0; h < kN / 4; ++h) {
+                w[h] = 0u;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) w[h] |= e4m3_of(v[k].x[4 * h + b], s) << (8 * b);
+            }
+            uint8_t* dst = qv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN;
+            if constexpr (kN == 4)
+                *reinterpret_cast<uint32_t*>(dst) = w[0];
+            else
+                *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+        }
     } else {
-        for (int64_t e = e0; e < total; ++e) q[e] = (uint8_t)e4m3_of(load_x(x, e), s[e / view_elems]);
+        const int64_t e1 = min(view_elems, e0 + piece_elems<T>());
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) qv[e] = (uint8_t)e4m3_of(load_x(xv, e), s);
     }
 }
 
@@ -90,27 +157,28 @@ extern "C" ludvig_status ludvig_fp8_quantize(const void* feats, int32_t dtype, i
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     LV_CUDA(cudaMemsetAsync(scales, 0, sizeof(float) * (size_t)n_views, st));
     if (view_elems > 0) {
-        const unsigned gx = (unsigned)std::min<int64_t>(ceil_div(view_elems, 256), 1024);
-        const dim3 grid(gx, (unsigned)n_views);
+        const int64_t piece = dtype == LUDVIG_F32 ? piece_elems<float>() : piece_elems<__nv_bfloat16>();
+        const int64_t pieces = ceil_div(view_elems, piece);
+        LV_ARG(pieces <= 0x7fffffff, "view too large");
+        const dim3 grid((unsigned)std::min<int64_t>(pieces, 1024), (unsigned)n_views);
+        const dim3 qgrid((unsigned)pieces, (unsigned)n_views);
+        const float* xf = static_cast<const float*>(feats);
+        const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(feats);
+        uint32_t* bits = reinterpret_cast<uint32_t*>(scales);
         if (dtype == LUDVIG_F32)
-            k_view_absmax<float><<<grid, 256, 0, st>>>(static_cast<const float*>(feats), view_elems,
-                                                       reinterpret_cast<uint32_t*>(scales));
+            k_view_absmax<float><<<grid, 256, 0, st>>>(xf, view_elems, bits);
         else
-            k_view_absmax<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(feats), view_elems,
-                                                               reinterpret_cast<uint32_t*>(scales));
+            k_view_absmax<__nv_bfloat16><<<grid, 256, 0, st>>>(xb, view_elems, bits);
         LV_LAUNCH();
-    }
-    k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
-    LV_LAUNCH();
-    const int64_t total = (int64_t)n_views * view_elems;
-    if (total > 0) {
-        const unsigned blocks = (unsigned)ceil_div(ceil_div(total, 4), 256);
+        k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
+        LV_LAUNCH();
         if (dtype == LUDVIG_F32)
-            k_quantize_e4m3<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(feats), scales, view_elems,
-                                                          total, q);
+            k_quantize_e4m3<float><<<qgrid, 256, 0, st>>>(xf, scales, view_elems, q);
         else
-            k_quantize_e4m3<__nv_bfloat16><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(feats), scales,
-                                                                  view_elems, total, q);
+            k_quantize_e4m3<__nv_bfloat16><<<qgrid, 256, 0, st>>>(xb, scales, view_elems, q);
+        LV_LAUNCH();
+    } else {
+        k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
         LV_LAUNCH();
     }
     return LUDVIG_OK;
