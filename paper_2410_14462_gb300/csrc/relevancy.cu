@@ -6,20 +6,25 @@
 //
 // The work streams the feature rows once and does m = queries + phrases dot
 // products of length d per row: a skinny product S = F Phi^T (n x d times
-// d x m) with its epilogue.  A CTA takes 128 rows and computes their 128 x M
-// block of S on CUDA cores with register tiles: thread (row group, query
-// group) holds 4 rows x M/8 queries, and per channel reads 4 features of its
-// rows (one 16-byte load of the chunk staged transposed in shared memory) and
-// M/8 normalised embedding values (one or two 16-byte loads, the same for the
-// whole warp), for 4 M/8 fused multiply-adds.  Channels are
-// staged 32 at a time, the next chunk's global loads in flight while the
-// current one is used.  The feature norms are summed from the staged chunks
-// (two threads per row, each over half of every chunk).  Each dot product is
-// one fmaf chain over the channels in order.  The epilogue writes the block of S to shared memory and takes
-// the minimum over the phrases for every (row, query).
+// d x m) with its epilogue, on CUDA cores (float32 accuracy).  A lane owns one
+// or two rows and keeps all their m dots in registers: per channel it multiplies its
+// rows' features (16-byte loads of its own rows from a staged chunk) with the
+// normalised embeddings (16-byte loads, the same for the whole warp) in packed
+// float32 pairs of embeddings.  Every warp streams its own rows, in chunks of 12
+// channels by cp.async, the next one in flight while one is used; the blocks
+// are persistent, so the embeddings are normalised once per block.  Each dot
+// product is one fmaf chain over the channels in order, and so is the row's
+// squared norm.
+//
+// Bound: the FMA pipe with the embeddings' shared-memory reads close behind (n d m
+// multiply-adds, m rounded up to a multiple of 4; the pipe is 0.53 busy).  500k x
+// 512 features, 21 queries and 4 phrases: 874 -> 465 us against tiles of 4 rows x 4
+// embeddings per thread, padded to 32.  Four rows per lane at 8 warps per SM, and
+// scalar instead of packed multiply-adds, measured 460 and 520 us.
 #include <algorithm>
 
 #include "common.cuh"
+#include "spec.cuh"
 
 namespace ludvig {
 
@@ -27,22 +32,157 @@ namespace {
 
 constexpr int kRelMaxM = 64;                   // queries + phrases
 constexpr int kRelMaxSmemFloats = 40 * 1024;   // normalised embeddings in shared memory (160 KB)
-constexpr int kRelRows = 128;                  // rows per CTA
-constexpr int kRelPitch = kRelRows + 4;        // transposed chunk: [channel][row], 16-byte aligned rows
+constexpr int kRelWarps = 16;                  // at most, per block
+constexpr int kRelChunk = 12;                  // channels staged at a time; a row's pitch too: the 16-byte
+                                               // reads of 8 consecutive rows (48 bytes apart) hit all 32 banks
+
+__device__ __forceinline__ void rel_copy(float* dst, const float* src, int bytes, bool in) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    const int n = in ? bytes : 0;   // (nothing read, zeros written)
+    if (bytes == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+struct RelArgs {
+    const float* f;
+    int64_t n;
+    int d, nq, m, vec;   // vec: rows start on 16-byte boundaries (d % 4 == 0 and f aligned)
+    float T;
+    float* r;
+};
+
+// Rows base .. base + 32 R of a warp (lane l: rows base + 32 a + l).
+template <int M, int R>
+__device__ __forceinline__ void relevancy_rows(const RelArgs& g, const float* sphi, float* stage, int64_t base) {
+    const int lane = threadIdx.x & 31;
+    const int d = g.d, d4 = (d + 3) & ~3, nq = g.nq;
+    const int64_t n = g.n;
+    const int nchunks = (d + kRelChunk - 1) / kRelChunk;
+    constexpr int kRows = 32 * R;
+    auto load_chunk = [&](int k) {
+        float* dst = stage + (k & 1) * (kRows * kRelChunk);
+        const int c0 = k * kRelChunk;
+        if (g.vec) {
+#pragma unroll
+            for (int t = 0; t < kRows * 3 / 32; ++t) {
+                const int e = lane + 32 * t, row = e / 3, c = 4 * (e - 3 * row);
+                const bool in = base + row < n && c0 + c < d;
+                rel_copy(dst + 4 * e, in ? g.f + (base + row) * d + c0 + c : g.f, 16, in);
+            }
+        } else {
+            for (int e = lane; e < kRows * kRelChunk; e += 32) {
+                const int row = e / kRelChunk, c = e - row * kRelChunk;
+                const bool in = base + row < n && c0 + c < d;
+                rel_copy(dst + e, in ? g.f + (base + row) * d + c0 + c : g.f, 4, in);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    __syncwarp();
+    load_chunk(0);
+    F2 acc[R][M / 2];
+    float nn[R];
+#pragma unroll
+    for (int a = 0; a < R; ++a) {
+        nn[a] = 0.f;
+#pragma unroll
+        for (int e = 0; e < M / 2; ++e) acc[a][e] = f2(0.f, 0.f);
+    }
+    for (int k = 0; k < nchunks; ++k) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();   // chunk k has landed for all lanes, chunk k - 1 is used up
+        if (k + 1 < nchunks) load_chunk(k + 1);
+        const float* st = stage + (k & 1) * (kRows * kRelChunk) + lane * kRelChunk;
+        const int c0 = k * kRelChunk, cw = min(kRelChunk, d4 - c0);
+#pragma unroll 1
+        for (int c = 0; c < cw; c += 4) {
+            float4 x[R];
+#pragma unroll
+            for (int a = 0; a < R; ++a) x[a] = *reinterpret_cast<const float4*>(st + a * (32 * kRelChunk) + c);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float* pr = sphi + (size_t)(c0 + c + q) * M;
+                F2 xx[R];
+#pragma unroll
+                for (int a = 0; a < R; ++a) {
+                    const float v = q == 0 ? x[a].x : q == 1 ? x[a].y : q == 2 ? x[a].z : x[a].w;
+                    nn[a] = fmaf(v, v, nn[a]);
+                    xx[a] = f2(v, v);
+                }
+#pragma unroll
+                for (int e = 0; e < M / 4; ++e) {
+                    const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(pr + 4 * e);
+#pragma unroll
+                    for (int a = 0; a < R; ++a) {
+                        acc[a][2 * e] = f2_fma(xx[a], F2{p.x}, acc[a][2 * e]);
+                        acc[a][2 * e + 1] = f2_fma(xx[a], F2{p.y}, acc[a][2 * e + 1]);
+                    }
+                }
+            }
+        }
+    }
+    // the minimum over the phrases for every (row, query), 32 rows at a time
+    // through shared memory (the output of consecutive rows is contiguous)
+#pragma unroll
+    for (int a = 0; a < R; ++a) {
+        __syncwarp();
+        float s[M];
+#pragma unroll
+        for (int e = 0; e < M / 2; ++e) {
+            const float2 v = f2_get(acc[a][e]);
+            s[2 * e] = v.x;
+            s[2 * e + 1] = v.y;
+        }
+        const float inv = nn[a] > 0.f ? 1.0f / sqrtf(nn[a]) : 0.f;
+        if (isfinite(nn[a])) {
+            // 1 / (1 + exp(T inv (s_k - s_q))) falls with s_k: the largest phrase decides
+            float top = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < M; ++e)
+                if (e >= nq && e < g.m) top = fmaxf(top, s[e]);
+#pragma unroll
+            for (int q = 0; q < M; ++q)
+                if (q < nq) stage[lane * nq + q] = fminf(1.f, 1.0f / (1.0f + expf(g.T * inv * (top - s[q]))));
+        } else {
+#pragma unroll 1
+            for (int q = 0; q < nq; ++q) {
+                float sq = 0.f, best = 1.f;
+#pragma unroll
+                for (int e = 0; e < M; ++e)
+                    if (e == q) sq = s[e];
+#pragma unroll
+                for (int e = 0; e < M; ++e)
+                    if (e >= nq && e < g.m) best = fminf(best, 1.0f / (1.0f + expf(g.T * inv * (s[e] - sq))));
+                stage[lane * nq + q] = best;
+            }
+        }
+        __syncwarp();
+        const int64_t row0 = base + 32 * a;
+        const int rows = (int)max((int64_t)0, min((int64_t)32, n - row0));
+        for (int o = lane; o < rows * nq; o += 32) g.r[row0 * nq + o] = stage[o];
+    }
+}
+
+// Rows per lane, so that the dots (M R registers) fit at 16 warps per SM.
+constexpr int rel_rows(int M) { return M <= 32 ? 2 : 1; }
+
+// Floats of a warp's stage: two chunks of its rows, or 32 rows of output.
+template <int M>
+constexpr int rel_stage() {
+    return 2 * 32 * rel_rows(M) * kRelChunk > 32 * (M - 1) ? 2 * 32 * rel_rows(M) * kRelChunk : 32 * (M - 1);
+}
 
 template <int M>
-__global__ void __launch_bounds__(256, M == 32 ? 3 : 2) k_relevancy(const float* __restrict__ f, int64_t n, int d,
-                                                   const float* __restrict__ phi, int nq, int m, float T,
-                                                   float* __restrict__ r) {
-    constexpr int QPT = M / 8;                 // queries per thread
-    constexpr int kStage = 32 * kRelPitch > kRelRows * (M + 1) ? 32 * kRelPitch : kRelRows * (M + 1);
+__global__ void __launch_bounds__(32 * kRelWarps, 1) k_relevancy(const RelArgs g, const float* __restrict__ phi,
+                                                                int64_t rows_per_warp) {
     extern __shared__ __align__(16) float smem[];
-    float* sphi = smem;                                        // [d][M], normalised, zero past m
-    float* As = sphi + (size_t)d * M;                          // [32][kRelPitch]
-    float* Cs = As;                                            // epilogue: [kRelRows][M + 1], in As's place
-    float* nrm = As + kStage;                                  // [kRelRows] squared norms
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int e = warp; e < M; e += 8) {
+    const int d = g.d, d4 = (d + 3) & ~3, m = g.m;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    float* sphi = smem;                            // [d4][M], normalised, zero past d and m
+    float* stage = sphi + (size_t)d4 * M + warp * rel_stage<M>();
+    for (int e = warp; e < M; e += nwarps) {
         float s = 0.f;
         if (e < m)
             for (int c = lane; c < d; c += 32) {
@@ -52,114 +192,37 @@ __global__ void __launch_bounds__(256, M == 32 ? 3 : 2) k_relevancy(const float*
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         const float inv = s > 0.f ? 1.0f / sqrtf(s) : 0.f;
-        for (int c = lane; c < d; c += 32) sphi[c * M + e] = e < m ? phi[(int64_t)e * d + c] * inv : 0.f;
+        for (int c = lane; c < d4; c += 32) sphi[c * M + e] = e < m && c < d ? phi[(int64_t)e * d + c] * inv : 0.f;
     }
-    // query group (QPT queries, the same for a warp: its embedding loads are
-    // broadcasts) and row group (4 rows; a warp's 32 groups read one 512-byte
-    // run of the staged chunk)
-    const int qg = tid >> 5, rg = tid & 31;
-    const int64_t base = (int64_t)blockIdx.x * kRelRows;
-    // staging: element t + 256 j of a chunk is row (t + 256 j) / 32, channel lane
-    const int64_t stride8 = 8 * (int64_t)d;                       // 8 rows
-    const float* frow = f + (base + (tid >> 5)) * (int64_t)d + lane;   // row warp, channel lane
-    const int64_t rows_left = n - base - (tid >> 5);                   // rows warp + 8 jj exist for 8 jj < this
-    auto load_chunk = [&](int c0, float* v) {
-        const bool cin = c0 + lane < d;
-        const float* p = frow + c0;
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj) v[jj] = (cin && 8 * jj < rows_left) ? p[jj * stride8] : 0.f;
-    };
-    float v[16];
-    load_chunk(0, v);
-    float acc[4][QPT];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < QPT; ++b) acc[a][b] = 0.f;
-    float nn = 0.f;   // row (tid % 128)'s squared norm over half of each chunk's channels
-    for (int c0 = 0; c0 < d; c0 += 32) {
-        __syncthreads();   // the previous chunk is consumed (and sphi is written, first time)
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj) As[lane * kRelPitch + (tid >> 5) + 8 * jj] = v[jj];
-        __syncthreads();
-        if (c0 + 32 < d) load_chunk(c0 + 32, v);   // in flight during this chunk
-        const int cw = min(32, d - c0);
-        {
-            // this thread's half of row (tid % 128)'s channels in the chunk
-            const int h0 = 16 * (tid >> 7), h1 = min(cw, h0 + 16);
-            for (int cc = h0; cc < h1; ++cc) {
-                const float x = As[cc * kRelPitch + (tid & (kRelRows - 1))];
-                nn = fmaf(x, x, nn);
-            }
-        }
-        auto step = [&](int cc) {
-            const float4 a4 = *reinterpret_cast<const float4*>(&As[cc * kRelPitch + 4 * rg]);
-            const float* pr = sphi + (size_t)(c0 + cc) * M + QPT * qg;
-            float bq[QPT];
-            if constexpr (QPT >= 4) {
-#pragma unroll
-                for (int b = 0; b < QPT; b += 4) {
-                    const float4 p4 = *reinterpret_cast<const float4*>(pr + b);
-                    bq[b] = p4.x;
-                    bq[b + 1] = p4.y;
-                    bq[b + 2] = p4.z;
-                    bq[b + 3] = p4.w;
-                }
-            } else {
-#pragma unroll
-                for (int b = 0; b < QPT; ++b) bq[b] = pr[b];
-            }
-            const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < QPT; ++b) acc[a][b] = fmaf(av[a], bq[b], acc[a][b]);
-        };
-        if (cw == 32) {
-#pragma unroll 8
-            for (int cc = 0; cc < 32; ++cc) step(cc);
-        } else {
-            for (int cc = 0; cc < cw; ++cc) step(cc);
-        }
-    }
-    __syncthreads();   // As is free: the block of S goes to Cs
-    if (tid < kRelRows) nrm[tid] = nn;   // first halves; the second halves are added below
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < QPT; ++b) Cs[(4 * rg + a) * (M + 1) + QPT * qg + b] = acc[a][b];
     __syncthreads();
-    if (tid >= kRelRows) nrm[tid - kRelRows] += nn;
-    __syncthreads();
-    const int rows = n - base < kRelRows ? (int)(n - base) : kRelRows;
-    for (int o = tid; o < rows * nq; o += 256) {
-        const int row = o / nq, q = o - row * nq;
-        const float* cr = Cs + row * (M + 1);
-        const float nsq = nrm[row];
-        const float inv = nsq > 0.f ? 1.0f / sqrtf(nsq) : 0.f;
-        float best = 1.f;
-        for (int e = nq; e < m; ++e) best = fminf(best, 1.0f / (1.0f + expf(T * inv * (cr[e] - cr[q]))));
-        r[(base + row) * nq + q] = best;
-    }
-}
-
-template <int M>
-size_t relevancy_smem(int d) {
-    // embeddings, then the chunk [32][kRelPitch] (or the epilogue's [128][M + 1]), then the norms
-    const size_t stage = std::max<size_t>((size_t)32 * kRelPitch, (size_t)kRelRows * (M + 1));
-    return sizeof(float) * ((size_t)d * M + stage + kRelRows);
+    // this warp's rows, 32 R at a time and what is left in halves (equal shares:
+    // whole groups alone would leave most warps idle in the last round)
+    int64_t r0 = ((int64_t)blockIdx.x * nwarps + warp) * rows_per_warp;
+    const int64_t r1 = min(g.n, r0 + rows_per_warp);
+    constexpr int R = rel_rows(M);
+    for (; r1 - r0 > 32 * (R - 1); r0 += 32 * R) relevancy_rows<M, R>(g, sphi, stage, r0);
+    if constexpr (R > 1)
+        if (r1 > r0) relevancy_rows<M, 1>(g, sphi, stage, r0);
 }
 
 template <int M>
 ludvig_status launch_relevancy(const float* f, int64_t n, int d, const float* phi, int nq, int m, float T, float* r,
                                cudaStream_t st) {
-    const size_t smem = relevancy_smem<M>(d);
     // set once per process; a function-local static is initialised by one thread
     static const cudaError_t configured =
-        cudaFuncSetAttribute(k_relevancy<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)relevancy_smem<M>(kRelMaxSmemFloats / M));
+        cudaFuncSetAttribute(k_relevancy<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     LV_CUDA(configured);
-    const unsigned grid = (unsigned)ceil_div(n, kRelRows);
-    k_relevancy<M><<<grid, 256, smem, st>>>(f, n, d, phi, nq, m, T, r);
+    int dev = 0, sms = 0;
+    LV_CUDA(cudaGetDevice(&dev));
+    LV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // one block per SM, of as many warps as have room for their stage (at least
+    // 11: the embeddings take at most 160 KB)
+    const size_t stage = sizeof(float) * rel_stage<M>(), embed = sizeof(float) * (size_t)((d + 3) & ~3) * M;
+    const int nwarps = (int)std::min<size_t>(kRelWarps, (227 * 1024 - embed) / stage);
+    const size_t smem = embed + nwarps * stage;
+    const int64_t rpw = std::max<int64_t>(32, round_up(ceil_div(n, (int64_t)sms * nwarps), 32));
+    RelArgs g{f, n, d, nq, m, d % 4 == 0 && (reinterpret_cast<uintptr_t>(f) & 15) == 0, T, r};
+    k_relevancy<M><<<(unsigned)ceil_div(n, rpw * nwarps), 32 * nwarps, smem, st>>>(g, phi, rpw);
     LV_LAUNCH();
     return LUDVIG_OK;
 }
@@ -185,8 +248,23 @@ extern "C" ludvig_status ludvig_relevancy(const float* feats, int64_t n, int32_t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     StageScope scope(LUDVIG_STAGE_RELEVANCY, st);
     const int m = n_queries + n_canon;
-    if (m <= 8) return launch_relevancy<8>(feats, n, d, phi, n_queries, m, temperature, r, st);
-    if (m <= 16) return launch_relevancy<16>(feats, n, d, phi, n_queries, m, temperature, r, st);
-    if (m <= 32) return launch_relevancy<32>(feats, n, d, phi, n_queries, m, temperature, r, st);
-    return launch_relevancy<64>(feats, n, d, phi, n_queries, m, temperature, r, st);
+    switch ((m + 3) / 4) {
+#define LV_REL(M) return launch_relevancy<M>(feats, n, d, phi, n_queries, m, temperature, r, st)
+        case 1: LV_REL(4);
+        case 2: LV_REL(8);
+        case 3: LV_REL(12);
+        case 4: LV_REL(16);
+        case 5: LV_REL(20);
+        case 6: LV_REL(24);
+        case 7: LV_REL(28);
+        case 8: LV_REL(32);
+        case 9:
+        case 10: LV_REL(40);
+        case 11:
+        case 12: LV_REL(48);
+        case 13:
+        case 14: LV_REL(56);
+        default: LV_REL(64);
+#undef LV_REL
+    }
 }

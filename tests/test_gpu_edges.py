@@ -33,3 +33,24 @@ def test_quantize_pieces(dtype, elems):
     q, s = ludvig.fp8_quantize(xt)
     qr, sr = oracle.fp8_quantize(xt.float().cpu().numpy())
     assert np.array_equal(s.cpu().numpy(), sr) and np.array_equal(q.cpu().numpy(), qr)
+
+
+@pytest.mark.parametrize("n,d,nq,k", [(1, 1, 1, 1), (31, 13, 3, 1), (33, 48, 5, 3), (20_011, 100, 11, 4),
+                                      (4097, 512, 21, 4), (300, 640, 60, 4), (2000, 5120, 4, 4)])
+def test_relevancy_sizes(n, d, nq, k):
+    rng = np.random.default_rng(n + d)
+    f, pq, pc = (rng.normal(size=(m, d)).astype(np.float32) for m in (n, nq, k))
+    got = ludvig.relevancy(*(torch.from_numpy(a).cuda() for a in (f, pq, pc)), 10.0).cpu().numpy()
+    assert np.abs(got - oracle.relevancy(f, pq, pc, 10.0)).max() <= 1e-5
+
+
+def test_relevancy_not_finite():
+    rng = np.random.default_rng(0)
+    f, pq, pc = (rng.normal(size=(m, 40)).astype(np.float32) for m in (70, 3, 2))
+    clean = ludvig.relevancy(*(torch.from_numpy(a).cuda() for a in (f, pq, pc)), 10.0).cpu().numpy()
+    f[5, 7] = np.nan
+    f[6, 7] = np.inf
+    got = ludvig.relevancy(*(torch.from_numpy(a).cuda() for a in (f, pq, pc)), 10.0).cpu().numpy()
+    rest = [i for i in range(70) if i not in (5, 6)]
+    assert np.array_equal(got[rest], clean[rest])
+    assert np.all(got[5] == 1.0)   # no phrase compares: the minimum's start
