@@ -54,3 +54,41 @@ def test_relevancy_not_finite():
     rest = [i for i in range(70) if i not in (5, 6)]
     assert np.array_equal(got[rest], clean[rest])
     assert np.all(got[5] == 1.0)   # no phrase compares: the minimum's start
+
+
+def _graph_ref(n, k, df, seed):
+    s = inputs.scene_clusters(n, seed=seed, n_clusters=5, sigma=0.05, extent=1.0)
+    f = np.random.default_rng(seed).normal(size=(n, df)).astype(np.float32)
+    f[::97] = 0.0
+    nbr, _ = oracle.knn(s.means, k)
+    return s, f, nbr, oracle.union_edges(nbr)
+
+
+@pytest.mark.parametrize("n,k,df", [(40, 3, 1), (20_000, 8, 127), (3000, 16, 128), (3000, 5, 132), (2000, 16, 390),
+                                    (2000, 33, 512), (1500, 4, 515)])
+def test_graph_widths(n, k, df):
+    s, f, nbr, (rows, cols) = _graph_ref(n, k, df, n + df)
+    sc = ludvig.Scene.from_inputs(s)
+    assert np.array_equal(ludvig.knn(sc, k).cpu().numpy(), nbr)
+    g = ludvig.Graph(sc, k, torch.from_numpy(f).cuda(), spatial_h=0.01, row_normalize=True)
+    _, col, val = (t.cpu().numpy() for t in g.export())
+    A = oracle.csr(n, rows, cols, oracle.edge_weights_spatial_cos(s.means, f, rows, cols, h=0.01))
+    assert np.array_equal(col, cols)
+    assert rel_l2(val, np.asarray(A[rows, cols]).ravel()) <= 1e-5
+
+
+@pytest.mark.parametrize("dx,scale", [(2, 1.0), (4, 1e-30), (5, 1e25), (17, 1.0), (32, 1e-12)])
+def test_diffusion_columns(dx, scale):
+    """Column remainders; the norms hold over the float32 range."""
+    s, f, _, (rows, cols) = _graph_ref(5000, 8, 16, dx)
+    sc = ludvig.Scene.from_inputs(s)
+    g = ludvig.Graph(sc, 8, torch.from_numpy(f).cuda(), spatial_h=0.01, row_normalize=True)
+    A = oracle.csr(5000, rows, cols, oracle.edge_weights_spatial_cos(s.means, f, rows, cols, h=0.01))
+    x = (np.random.default_rng(dx).random((5000, dx)) * scale).astype(np.float32)
+    x[:, 0] = 0.0
+    for steps, gate in ((1, 1e-5), (6, 1e-4)):
+        got = g.diffuse(torch.from_numpy(x).cuda(), steps).cpu().numpy()
+        ref = oracle.diffuse(A, x, steps)
+        assert np.all(got[:, 0] == 0.0)
+        for c in range(1, dx):
+            assert rel_l2(got[:, c], ref[:, c]) <= gate
