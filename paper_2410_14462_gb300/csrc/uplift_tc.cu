@@ -88,7 +88,7 @@ struct WeightsArgs {
     int64_t npad;
     const uint2* ranges;
     int ntiles, TX, width, height;
-    uint8_t* wg1;           // [cap][128][256] bfloat16: W (NT = 1) or W1
+    uint8_t* wg1;           // [cap][128][256] bfloat16: W (NT = 1) or W1; float32: W (NT = 3)
     uint8_t* wg2;           // W2 (NT = 2)
     uint32_t* chunk_gid;    // [cap][128]
     int* chunk_rows;        // [cap]
@@ -96,7 +96,7 @@ struct WeightsArgs {
     int* item_first;        // [nitems]: the tile's first chunk, or -1 (set to -1 before the launch)
     int* chunk_counter;
     int cap;
-    float* chunk_den;       // [cap][128][NT]: each row's den, the sum of its weight terms, in term 0's
+    float* chunk_den;       // [cap][128][1, or 2 for NT = 2]: each row's den, the sum of its weight terms, in term 0's
                             // slot (term 1's: 0); rewritten on a re-run
     // direct accumulation (k_weights<NT, true>, few channels): each new row's
     // sum_p w F[p, c] and its den go straight into the view's num and den
@@ -109,6 +109,7 @@ struct WeightsArgs {
 
 constexpr int kDirectMaxD = 4;
 constexpr int kQuadItems = 152 * 16;
+constexpr int kBlockItems = 152 * 12;   // below: weight rows by blocks of 8 warps per tile
 
 __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int rows, int next) {
     if (c >= 0 && c < a.cap) {
@@ -120,6 +121,7 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
 // The weights of one (view, tile), a warp per tile (NB = 4) or per 8x8 quadrant
 // of it (NB = 1); a lane holds two neighbouring pixels of each quadrant.
 //   DD = 0: weight rows; DD = 1 .. 4: direct accumulation of DD channels.
+//   NT = 1, 2: weights as one or two bfloat16 terms; 3: float32 rows.
 //   COUNT: den is the number of a row's non-zero weights instead of their sum.
 //
 // Bound: instruction issue (0.74 of it, FMA pipe and ALU half busy each), with
@@ -145,9 +147,11 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
 template <int NT, int DD, int NB, bool COUNT>
 __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_constant__ WeightsArgs a) {
     constexpr bool kDirect = DD > 0;
+    constexpr int kPx = NT == 3 ? 4 : 2;           // bytes per pixel of a row
+    constexpr int kDen = NT == 2 ? 2 : 1;          // den slots per row
     constexpr int kVals = kDirect ? DD + 1 : 1;   // sums per row
     constexpr int kRowBuf = 32 / kVals;           // rows whose lane sums are kept
-    constexpr int kGroup = NB == 1 ? 2 : 1;       // entries taken together
+    constexpr int kGroup = NB == 1 ? 2 : 1;       // entries taken together (a row is one entry's: NB = 4 takes one)
     constexpr uint32_t kAll = 0xffffffffu;
     __shared__ float4 s_rec[32][3];               // the batch's records, every value twice
     __shared__ float s_part[32 * 33];             // [row][sum][lane]
@@ -225,7 +229,7 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
     float* const vden = kDirect ? a.views.den[v] : nullptr;
     // sum `i` of the kept rows over the lanes
     // byte of quadrant b's first pixel in a row
-    auto kQuadByte = [](int b) { return (b >> 1) * 256 + (b & 1) * 16; };
+    auto kQuadByte = [](int b) { return ((b >> 1) * 128 + (b & 1) * 8) * kPx; };
     auto lane_sum = [&](int i) {
         const float* p = s_part + 33 * i;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -315,7 +319,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                     local = 0;
                     // (a launch that runs out of chunks is redone: what it
                     // writes to the last one is not used)
-                    const size_t o = (size_t)min(cur, a.cap - 1) * kChunkBytes + (lane >> 2) * 32 + (lane & 3) * 4;
+                    const size_t o =
+                        (size_t)min(cur, a.cap - 1) * (kCRows * 256 * kPx) + ((lane >> 2) * 16 + (lane & 3) * 2) * kPx;
                     d1 = a.wg1 + o;
                     if (NT == 2) d2 = a.wg2 + o;
                 }
@@ -347,7 +352,9 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                         const float wx = tn.x >= kTransMin ? ww.x : 0.f, wy = tn.y >= kTransMin ? ww.y : 0.f;
                         nz |= __float_as_uint(wx) | __float_as_uint(wy);
                         F2 wv = f2(wx, wy);
-                        if (!kDirect || NT == 1) {
+                        if (NT == 3) {
+                            *reinterpret_cast<float2*>(d1 + kQuadByte(b)) = make_float2(wx, wy);
+                        } else if (!kDirect || NT == 1) {
                             const __nv_bfloat162 h = __floats2bfloat162_rn(wx, wy);
                             const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
                             const F2 hf = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u));
@@ -375,6 +382,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                         auto quad_or_zero = [&](int b) {
                             if (B[b] & bit) {
                                 finish(b, alpha(g, b));
+                            } else if (NT == 3) {
+                                *reinterpret_cast<float2*>(d1 + kQuadByte(b)) = make_float2(0.f, 0.f);
                             } else if (!kDirect) {
                                 *reinterpret_cast<uint32_t*>(d1 + kQuadByte(b)) = 0u;
                                 if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + kQuadByte(b)) = 0u;
@@ -410,8 +419,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                         rowbits |= bit;
                         ++nbuf;
                         ++local;
-                        d1 += kRowBytes;
-                        if (NT == 2) d2 += kRowBytes;
+                        d1 += 256 * kPx;
+                        if (NT == 2) d2 += 256 * kPx;
                     }
                 }
             }
@@ -435,8 +444,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
             if (((rowbits >> lane) & 1u) && myrow >= 0) {
                 const float s = lane_sum(__popc(rowbits & lt_mask));
                 // the row's den in term 0's slot (the aggregation adds the slots)
-                a.chunk_den[(size_t)myrow * NT] = s;
-                if (NT == 2) a.chunk_den[(size_t)myrow * NT + 1] = 0.f;
+                a.chunk_den[(size_t)myrow * kDen] = s;
+                if (NT == 2) a.chunk_den[(size_t)myrow * kDen + 1] = 0.f;
                 a.chunk_gid[myrow] = gid;
             }
             nbuf = 0;
@@ -446,6 +455,286 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
         if (nbuf > 0) flush_direct();
     } else {
         if (lane == 0 && cur >= 0) finish_chunk(a, cur, local, -1);
+    }
+}
+
+// The weight rows of launches with few tiles: a block of 8 warps per tile, one
+// 8x4 pixel block per warp, a pixel per lane.  k_weights issues half as many
+// instructions, but a warp alone issues one every four or five cycles, so where the
+// tiles do not fill the schedulers the longest tile's walk is the time, and here
+// eight warps share it.  320x240 views of 100k clustered (uniform)
+// Gaussians, float32: 1200 tiles 386 (256) us against k_weights' 574 (286), 2400 tiles 528 (405)
+// against 634 (336), 4800 tiles 920 (705) against 819 (508).
+//
+// Batches of 32 entries: warp 0 gathers their records by cp.async kRing - 1
+// batches ahead and computes their block masks; the weights go to 32 staging rows
+// in shared memory, and the rows with a non-zero weight are then appended to the
+// tile's chunks.
+constexpr int kTcBatch = 32;   // Gaussians composited per step
+constexpr int kRing = 8;       // list-record batches in flight
+
+template <int NT>
+struct BlockSmem {
+    alignas(16) PairRec rec[kRing][kTcBatch];
+    alignas(16) uint8_t stage[NT][kTcBatch * kRowBytes];   // [term][j][256 pixels]
+    uint32_t rowmask[2];
+    int cur_chunk, cur_start, next_chunk;
+};
+
+// A weight row's contribution to den, from its 256 bfloat16 values (8 per
+// lane, packed in wv), summed over the warp: the sum of the term's values, or
+// with count_den the number of non-zero weights (counted on term 0; a weight
+// w > 0 is at least 1/255 * 1e-4, far above the smallest bfloat16).
+__device__ __forceinline__ float lane_den(const uint32_t* wv, bool count_den, int term) {
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (count_den)
+            s += term == 0 ? (float)((wv[k] & 0xffffu) != 0u) + (float)((wv[k] >> 16) != 0u) : 0.f;
+        else
+            s += __uint_as_float(wv[k] << 16) + __uint_as_float(wv[k] & 0xffff0000u);
+    }
+    return s;
+}
+
+__device__ __forceinline__ float warp_sum(float s) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+__device__ __forceinline__ float row_den(const uint32_t* wv, bool count_den, int term) {
+    return warp_sum(lane_den(wv, count_den, term));
+}
+
+template <int NT, bool COUNT>
+__global__ void __launch_bounds__(256, 5) k_weights_block(const __grid_constant__ WeightsArgs a) {
+    __shared__ BlockSmem<NT> S;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    const int item = blockIdx.x;
+    const int v = item / a.ntiles, tile = item - v * a.ntiles;
+    const int tx = tile % a.TX, ty = tile / a.TX;
+    const uint2 range = a.ranges[item];
+    const uint32_t nb = (range.y - range.x + kTcBatch - 1) / kTcBatch;
+    if (nb == 0) return;
+    // warp w covers the 8x4 pixel block ((w & 1) * 8, (w >> 1) * 4) of the tile
+    const int lx = (warp & 1) * 8 + (lane & 7), ly = (warp >> 1) * 4 + (lane >> 3);
+    const int pix = ly * kTile + lx;
+    const int px = tx * kTile + lx, py = ty * kTile + ly;
+    const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
+
+    if (tid == 0) {
+        S.rowmask[0] = 0u;
+        S.rowmask[1] = 0u;
+        S.cur_chunk = -1;
+        S.cur_start = 0;
+        S.next_chunk = -1;
+    }
+    for (int e = tid; e < (int)(NT * kTcBatch * kRowBytes / 16); e += 256)
+        reinterpret_cast<uint4*>(&S.stage[0][0])[e] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+
+    // batch k of the list goes to ring slot k % kRing.  Warp 0, lane j gathers
+    // entry j of a batch (two 16-byte cp.async of its 32-byte record) and
+    // commits one cp.async group per batch, empty past the list's end, so
+    // that "at most kRing - 2 groups pending" always means "batch k landed".
+    // The rank of the batch after next is loaded one iteration early, so the
+    // gather does not wait on it.
+    const PairRec* vrec = a.srec + (int64_t)v * a.npad;
+    auto rank_of = [&](uint32_t k) -> uint32_t {
+        const uint32_t e = range.x + k * kTcBatch + (uint32_t)lane;
+        return (k < nb && e < range.y) ? a.rank[e] : 0xffffffffu;
+    };
+    auto issue_records = [&](uint32_t k, uint32_t rk) {
+        if (warp == 0) {
+            if (rk != 0xffffffffu) {
+                PairRec* dst = &S.rec[k % kRing][lane];
+                cp_async_16(dst, vrec + rk);
+                cp_async_16(reinterpret_cast<uint8_t*>(dst) + 16, reinterpret_cast<const uint8_t*>(vrec + rk) + 16);
+            }
+            cp_async_commit();
+        }
+    };
+    uint32_t next_rank = 0xffffffffu;   // warp 0: rank of batch k + kRing - 1 at iteration k
+    // warp 0, lane j: entry j of batch k has landed; its block mask.  Batch 0's
+    // is computed here, batch k + 1's after warp 0 has composited batch k (off
+    // the path of the other warps, which are still compositing batch k)
+    auto mask_batch = [&](uint32_t k) {
+        cp_async_wait<kRing - 2>();
+        if (k < nb && range.x + k * kTcBatch + (uint32_t)lane < range.y) {
+            PairRec& r = S.rec[k % kRing][lane];
+            r.mask = block_mask_fast(r.mx, r.my, r.ca, r.cb, r.cc, r.op, tx, ty);
+        }
+    };
+    if (warp == 0) {
+        for (uint32_t k = 0; k + 1 < (uint32_t)kRing; ++k) issue_records(k, rank_of(k));
+        next_rank = rank_of(kRing - 1);
+        mask_batch(0);
+    }
+
+    float T = 1.0f;
+    bool done = !(px < a.width && py < a.height);
+    int nrows = 0;   // rows of this tile written so far
+    int buf = 0;
+    for (uint32_t k = 0; k < nb; ++k, buf ^= 1) {
+        const uint32_t slot = k % kRing;
+        if (__syncthreads_count(!done) == 0) break;
+        // every thread is past batch k-1: its slot takes batch k + kRing - 1
+        if (warp == 0) {
+            issue_records(k + kRing - 1, next_rank);
+            next_rank = rank_of(k + kRing);
+        }
+        if (tid == 0) {
+            // rows [nrows, nrows + 32) must have chunks; a chunk filled to
+            // exactly 128 rows may not have its successor yet
+            if (nrows >= S.cur_start + kCRows) {
+                if (S.next_chunk < 0) S.next_chunk = atomicAdd(a.chunk_counter, 1);
+                finish_chunk(a, S.cur_chunk, kCRows, S.next_chunk);
+                S.cur_chunk = S.next_chunk;
+                S.cur_start += kCRows;
+                S.next_chunk = -1;
+            }
+            if (S.cur_chunk < 0) {
+                S.cur_chunk = atomicAdd(a.chunk_counter, 1);
+                a.item_first[item] = S.cur_chunk;
+            }
+            if (nrows + kTcBatch > S.cur_start + kCRows && S.next_chunk < 0)
+                S.next_chunk = atomicAdd(a.chunk_counter, 1);
+        }
+        const PairRec* rec = S.rec[slot];
+        const int cnt = (int)min((uint32_t)kTcBatch, range.y - (range.x + k * kTcBatch));
+        uint32_t lm = 0u;   // this lane's non-zero weights (bit j = Gaussian j)
+        if (__any_sync(0xffffffffu, !done)) {
+            // Gaussians of the batch that can reach this warp's pixel block,
+            // four at a time in list order: the four alphas are independent,
+            // the transmittance recursion then takes them in order
+            uint32_t rel = __ballot_sync(0xffffffffu, lane < cnt && ((rec[lane].mask >> warp) & 1u));
+            while (rel != 0u && __any_sync(0xffffffffu, !done)) {
+                int jj[4];
+                float al[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    jj[q] = rel ? __ffs(rel) - 1 : -1;
+                    rel &= rel - 1u;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int j = jj[q] < 0 ? jj[0] : jj[q];
+                    const float4 g = *reinterpret_cast<const float4*>(&rec[j].mx);
+                    const float2 h = *reinterpret_cast<const float2*>(&rec[j].cc);
+                    al[q] = alpha_at_nb(g.x, g.y, g.z, g.w, h.x, h.y, pxf, pyf);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (jj[q] >= 0 && al[q] > 0.f && !done) {
+                        const float Tn = __fmul_rn(T, __fsub_rn(1.0f, al[q]));
+                        if (Tn < kTransMin) {
+                            done = true;
+                        } else {
+                            const float wv = __fmul_rn(al[q], T);
+                            T = Tn;
+                            lm |= 1u << jj[q];
+                            const int o = jj[q] * kRowBytes + pix * 2;
+                            const __nv_bfloat16 h1 = __float2bfloat16_rn(wv);
+                            *reinterpret_cast<__nv_bfloat16*>(&S.stage[0][o]) = h1;
+                            if (NT == 2)
+                                *reinterpret_cast<__nv_bfloat16*>(&S.stage[NT - 1][o]) =
+                                    __float2bfloat16_rn(wv - __bfloat162float(h1));
+                        }
+                    }
+                }
+            }
+            const uint32_t mine = __reduce_or_sync(0xffffffffu, lm);
+            if (lane == 0 && mine) atomicOr(&S.rowmask[buf], mine);
+        }
+        if (warp == 0) mask_batch(k + 1);   // (pending: batches k+1 .. k+kRing-1)
+        if (tid == 0) S.rowmask[buf ^ 1] = 0u;
+        __syncthreads();
+        const uint32_t rowmask = S.rowmask[buf];
+        const int nnew = __popc(rowmask);
+        const int cur = S.cur_chunk, nxt = S.next_chunk, cstart = S.cur_start;
+        // the staging row of the i-th new Gaussian (the i-th set bit j of the
+        // row mask) goes to tile row nrows + i (chunk cur, or nxt past its 128
+        // rows), 16 bytes per lane, one warp per row and term; the staging row
+        // is cleared behind, the row's sum of each term (the bfloat16 values the
+        // product uses) is kept for den, and the Gaussian id is recorded
+        if constexpr (NT == 2) {
+            // warp i % 8 takes row i, both terms
+            uint32_t m = rowmask;
+            for (int i = 0; m != 0u; ++i, m &= m - 1u) {
+                if ((i & 7) != warp) continue;
+                const int j = __ffs(m) - 1;
+                int local = nrows + i - cstart, ch = cur;
+                if (local >= kCRows) {
+                    local -= kCRows;
+                    ch = nxt;
+                }
+                const bool keep = ch >= 0 && ch < a.cap;
+                float sden = 0.f;   // this lane's part of the row's den, both terms
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                    uint4* src = reinterpret_cast<uint4*>(&S.stage[t][j * kRowBytes + lane * 16]);
+                    const uint4 v4 = *src;
+                    if (keep) {
+                        uint8_t* dst = (t == 0 ? a.wg1 : a.wg2) + (size_t)ch * kChunkBytes + local * kRowBytes + lane * 16;
+                        *reinterpret_cast<uint4*>(dst) = v4;
+                    }
+                    *src = make_uint4(0u, 0u, 0u, 0u);
+                    const uint32_t wv[4] = {v4.x, v4.y, v4.z, v4.w};
+                    sden += lane_den(wv, COUNT, t);
+                }
+                sden = warp_sum(sden);
+                if (lane == 0 && keep) {
+                    // the row's den in term 0's slot (the aggregation adds the slots)
+                    a.chunk_den[((size_t)ch * kCRows + local) * NT] = sden;
+                    a.chunk_den[((size_t)ch * kCRows + local) * NT + 1] = 0.f;
+                    a.chunk_gid[(size_t)ch * kCRows + local] = rec[j].gid;
+                }
+            }
+        } else {
+            // warp w takes row w (row i of the 32 at most: warp i % 8 on pass i / 8)
+            for (int e = tid; e < nnew * 32; e += 256) {
+                const int i = e >> 5;
+                const int j = (int)__fns(rowmask, 0u, i + 1);
+                int local = nrows + i - cstart, ch = cur;
+                if (local >= kCRows) {
+                    local -= kCRows;
+                    ch = nxt;
+                }
+                uint4* src = reinterpret_cast<uint4*>(&S.stage[0][j * kRowBytes + lane * 16]);
+                const uint4 v4 = *src;
+                if (ch >= 0 && ch < a.cap)
+                    *reinterpret_cast<uint4*>(a.wg1 + (size_t)ch * kChunkBytes + local * kRowBytes + lane * 16) = v4;
+                *src = make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t wv[4] = {v4.x, v4.y, v4.z, v4.w};
+                const float sden = row_den(wv, COUNT, 0);
+                if (lane == 0 && ch >= 0 && ch < a.cap) a.chunk_den[(size_t)ch * kCRows + local] = sden;
+            }
+            if (tid < kTcBatch && ((rowmask >> tid) & 1u)) {
+                int local = nrows + __popc(rowmask & lt_mask) - cstart, ch = cur;
+                if (local >= kCRows) {
+                    local -= kCRows;
+                    ch = nxt;
+                }
+                if (ch >= 0 && ch < a.cap) a.chunk_gid[(size_t)ch * kCRows + local] = rec[tid].gid;
+            }
+        }
+        nrows += nnew;
+        // no barrier here: the next batch's counting barrier orders these stores
+    }
+    // gathers issued past an early stop still land before the CTA exits
+    if (warp == 0) cp_async_wait<0>();
+    __syncthreads();
+    if (tid == 0) {
+        const int cur = S.cur_chunk, cstart = S.cur_start, nxt = S.next_chunk;
+        if (nrows > cstart + kCRows) {   // the last batch spilled into nxt
+            finish_chunk(a, cur, kCRows, nxt);
+            finish_chunk(a, nxt, nrows - cstart - kCRows, -1);
+        } else {
+            finish_chunk(a, cur, nrows - cstart, -1);
+            finish_chunk(a, nxt, 0, -1);   // allocated, never used
+        }
     }
 }
 
@@ -1542,7 +1831,7 @@ ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap) {
         void* q;
         LV_TRY(ws.get(kWsCounter[p], sizeof(int), &q));
         LV_TRY(ws.get(kWsFirst[p], sizeof(int) * (size_t)nitems, &q));
-        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes, &q));
+        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes * (NT == 3 ? 2 : 1), &q));
         if (NT == 2) LV_TRY(ws.get(kWsW2[p], (size_t)cap * kChunkBytes, &q));
         LV_TRY(ws.get(kWsGid[p], sizeof(uint32_t) * (size_t)cap * kCRows, &q));
         LV_TRY(ws.get(kWsRows[p], sizeof(int) * (size_t)cap, &q));
@@ -1553,6 +1842,20 @@ ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap) {
     }
     return LUDVIG_OK;
 }
+
+namespace {
+template <int NT>
+void launch_weight_rows(const WeightsArgs& w, int nitems, cudaStream_t st) {
+    const bool count = option_count_normalise();
+    if constexpr (NT != 3) {
+        if (nitems < kBlockItems) {
+            count ? k_weights_block<NT, true><<<nitems, 256, 0, st>>>(w) : k_weights_block<NT, false><<<nitems, 256, 0, st>>>(w);
+            return;
+        }
+    }
+    count ? k_weights<NT, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<NT, 0, 4, false><<<nitems, 32, 0, st>>>(w);
+}
+}  // namespace
 
 ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int NT, Arena& ws, int parity,
                          int* status, int64_t* chunk_cap, bool checked, cudaStream_t st, TileWeights* tw) {
@@ -1574,7 +1877,7 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
             set_error("tile weights need %lld chunks of 128 rows", (long long)cap);
             return LUDVIG_ERR_UNSUPPORTED;
         }
-        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes, &t.wg1));
+        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes * (NT == 3 ? 2 : 1), &t.wg1));
         if (NT == 2) LV_TRY(ws.get(kWsW2[p], (size_t)cap * kChunkBytes, &t.wg2));
         LV_TRY(ws.get(kWsGid[p], (size_t)cap * kCRows, &t.cgid));
         LV_TRY(ws.get(kWsRows[p], (size_t)cap, &t.crows));
@@ -1602,11 +1905,12 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         w.chunk_den = t.cden;
         w.one = make_float2(1.f, 1.f);
         const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
-        const bool count = option_count_normalise();
-        if (NT == 2)
-            count ? k_weights<2, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<2, 0, 4, false><<<nitems, 32, 0, st>>>(w);
+        if (NT == 3)
+            launch_weight_rows<3>(w, nitems, st);
+        else if (NT == 2)
+            launch_weight_rows<2>(w, nitems, st);
         else
-            count ? k_weights<1, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<1, 0, 4, false><<<nitems, 32, 0, st>>>(w);
+            launch_weight_rows<1>(w, nitems, st);
         LV_LAUNCH();
         trace_end(tslot, st);
         if (!checked) break;

@@ -25,6 +25,59 @@ def _lib():
     ludvig.load()
 
 
+def _uplift_error(wl, dtype, count=False):
+    sc = ludvig.Scene.from_inputs(wl.scene)
+    F = device_features(wl, range(wl.cams.v), dtype=dtype)
+    old = ludvig.get_option(ludvig.OPT_COUNT_NORMALISE)
+    ludvig.set_option(ludvig.OPT_COUNT_NORMALISE, int(count))
+    try:
+        out, beta = ludvig.uplift(sc, wl.cams.params, wl.cams.width, wl.cams.height, F)
+    finally:
+        ludvig.set_option(ludvig.OPT_COUNT_NORMALISE, old)
+    ref, bref = oracle.uplift(wl.scene, wl.cams, lambda v: F[v].float(), count_normalise=count)
+    pos = bref > 0
+    assert np.array_equal(beta.cpu().numpy() > 0, pos)
+    if count:
+        assert np.array_equal(beta.cpu().numpy(), bref)
+    return rel_l2(out.cpu().numpy(), ref, pos)
+
+
+# 5 views of 30 x 17 tiles: 2550 items, above the few-tile kernels' limits
+@pytest.mark.parametrize("d,dtype,gate,count", [(1, torch.float32, 1e-5, False), (3, torch.bfloat16, 1e-2, False),
+                                                (4, torch.float32, 1e-5, True), (40, torch.float32, 1e-5, False),
+                                                (40, torch.bfloat16, 1e-2, False), (48, torch.float32, 1e-5, True)])
+def test_many_tiles(d, dtype, gate, count):
+    wl = inputs.small_field_workload(n=6000, views=5, d=d, width=475, height=269)
+    assert _uplift_error(wl, dtype, count) <= gate
+
+
+# weights of the CUDA-core path are float32, so bfloat16 features meet the float32 bar
+@pytest.mark.parametrize("d,dtype,count", [(33, torch.float32, False), (100, torch.float32, False),
+                                           (101, torch.bfloat16, False), (132, torch.float32, True),
+                                           (516, torch.bfloat16, False), (520, torch.float32, False)])
+def test_cuda_core_widths(d, dtype, count):
+    wl = inputs.small_field_workload(n=20_000, views=2, d=d, width=83, height=61)
+    assert _uplift_error(wl, dtype, count) <= 1e-5
+
+
+def test_cuda_core_features_not_finite():
+    """A Gaussian without weight at a pixel does not see what the pixel holds."""
+    wl = inputs.small_field_workload(n=3000, views=1, d=33, width=83, height=61)
+    sc = ludvig.Scene.from_inputs(wl.scene)
+    F = device_features(wl, [0])
+    out, _ = ludvig.uplift(sc, wl.cams.params, 83, 61, F)
+    hit = torch.zeros((1, 61, 83, 1), device="cuda")
+    hit[0, 30, 40] = 1.0
+    touched, _ = ludvig.uplift(sc, wl.cams.params, 83, 61, hit)
+    F[0, 30, 40] = float("nan")
+    F[0, 30, 40, 1] = float("inf")
+    bad, _ = ludvig.uplift(sc, wl.cams.params, 83, 61, F)
+    t = touched[:, 0] > 0
+    assert t.any() and torch.isnan(bad[t][:, 0]).all()
+    assert torch.isfinite(bad[~t]).all()
+    assert rel_l2(bad[~t].cpu().numpy(), out[~t].cpu().numpy()) <= 1e-5
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("elems", [1, 4096, 8192 + 5, 16384])
 def test_quantize_pieces(dtype, elems):
