@@ -101,7 +101,6 @@ ludvig_scene* take_context(int dev) {
     ludvig_scene* c = new (std::nothrow) ludvig_scene();
     if (c) {
         c->device = dev;
-        c->onesweep = true;   // many groups: one kernel per radix pass
     }
     return c;
 }

@@ -994,12 +994,7 @@ ludvig_status front_end(ludvig_scene* ctx, const GroupViews& g, int width, int h
 
     uint32_t *sk = keys, *sv = vals;
     tslot = trace_on() ? trace_begin(LUDVIG_STAGE_DEPTH_SORT, st) : -1;
-    // (a packed batch's context sorts in one kernel per pass: fewer launches for
-    // many groups; a single call takes the faster reduce-then-scan passes)
-    if (s->onesweep)
-        LV_TRY(radix_sort_onesweep(&sk, &sv, keys2, vals2, nv, npad, nullptr, 32, s->dstat, ws, st));
-    else
-        LV_TRY(radix_sort_pairs(&sk, &sv, keys2, vals2, nv, npad, 32, ws, st));
+    LV_TRY(radix_sort_pairs(&sk, &sv, keys2, vals2, nv, npad, 32, ws, st));
     trace_end(tslot, st);
     tslot = trace_on() ? trace_begin(LUDVIG_STAGE_BIN, st) : -1;
     k_sorted_records<<<grid_for(nG, 256), 256, 0, st>>>(sk, sv, ntile, prec, n, npad, nG, cnt, srec,
@@ -1030,7 +1025,7 @@ ludvig_status front_end(ludvig_scene* ctx, const GroupViews& g, int width, int h
     LV_TRY(ws.get("up.pv2", (size_t)cap, &pv2));
     // 16-bit keys when the caller reads only the ranks and lists afterwards
     // (the tensor-core path) and every key and the sentinel fit
-    const bool k16 = keys16_ok && !s->onesweep && sentinel < 0xffffu && !dbg;
+    const bool k16 = keys16_ok && sentinel < 0xffffu && !dbg;
     if (k16)
         k_emit_pairs<uint16_t><<<grid_for(nG, kEmitThreads), kEmitThreads, 0, st>>>(cnt, off, srec, srect, npad, nG, TX, ntiles, prune,
                                                                   total_d, (uint64_t)cap, ovf, sentinel,
@@ -1048,8 +1043,6 @@ ludvig_status front_end(ludvig_scene* ctx, const GroupViews& g, int width, int h
     if (k16)
         LV_TRY(radix_sort_pairs_len16(&spk16, &spv, reinterpret_cast<uint16_t*>(pk2), pv2, 1, cap, total_d, nbits, ws,
                                       st));
-    else if (s->onesweep)
-        LV_TRY(radix_sort_onesweep(&spk, &spv, pk2, pv2, 1, cap, total_d, nbits, s->dstat, ws, st));
     else
         LV_TRY(radix_sort_pairs_len(&spk, &spv, pk2, pv2, 1, cap, total_d, nbits, ws, st));
     uint2* ranges;
@@ -1330,13 +1323,7 @@ ludvig_status reserve_async(ludvig_scene* s, int nv, int ng, int64_t n, int widt
     // up to n Gaussians) and their scan sums
     const int64_t npad = round_up(std::max<int64_t>(n, 1), kRadixTile);
     const int64_t hist = 256 * std::max<int64_t>(cap, (int64_t)ng * npad) / kRadixTile;
-    if (s->onesweep) {
-        LV_TRY(ws.get("os.status", sizeof(uint64_t) * (size_t)hist, &q));
-        LV_TRY(ws.get("os.hist", sizeof(uint32_t) * 4 * 256 * (size_t)std::max(ng, 1), &q));
-        LV_TRY(ws.get("os.counters", sizeof(uint32_t) * 4, &q));
-    } else {
-        LV_TRY(ws.get("radix.hist", sizeof(uint32_t) * (size_t)hist, &q));
-    }
+    LV_TRY(ws.get("radix.hist", sizeof(uint32_t) * (size_t)hist, &q));
     LV_TRY(ws.get("scan.sums", sizeof(unsigned long long) * (size_t)ceil_div(std::max(hist, (int64_t)ng * npad), 4096),
                   &q));
     const int TX = (width + kTile - 1) / kTile, TY = (height + kTile - 1) / kTile;
