@@ -1310,12 +1310,13 @@ ludvig_status run_checked_range(ludvig_scene* s, const ludvig_camera* cams, int 
 }
 
 // Allocates what asynchronous groups of up to nv views use at the scene's
-// current capacities (both buffer sets), so that they find it in place: a
+// current capacities, so that they find it in place: a
 // workspace that grows synchronises the device.
 // Groups of up to nv views whose largest per-view Gaussian scratch is that of
 // ng views of n Gaussians.
+// sets: the buffer sets that alternate between groups (one for a single group).
 ludvig_status reserve_async(ludvig_scene* s, int nv, int ng, int64_t n, int width, int height, const FeatSrc& src,
-                            bool tc) {
+                            bool tc, int sets) {
     Arena& ws = s->ws;
     void* q;
     FrontBufs fb;
@@ -1333,9 +1334,9 @@ ludvig_status reserve_async(ludvig_scene* s, int nv, int ng, int64_t n, int widt
     const bool padded = src_padded(src);
     const int fdt = src.kind == 2 ? LUDVIG_BF16 : src.dtype;
     const bool direct = src_direct(src);   // no weight rows, no padded copy
-    if (!direct) LV_TRY(tc_reserve(ws, !tc ? 3 : fdt == LUDVIG_F32 ? 2 : 1, nv * TX * TY, s->tc_chunk_cap));
+    if (!direct) LV_TRY(tc_reserve(ws, !tc ? 3 : fdt == LUDVIG_F32 ? 2 : 1, nv * TX * TY, s->tc_chunk_cap, sets));
     const int64_t npx = (int64_t)nv * width * height;
-    for (int p = 0; p < 2; ++p) {
+    for (int p = 0; p < sets; ++p) {
         static const char* const kFb[2] = {"fp8.bf16.0", "fp8.bf16.1"};
         static const char* const kPad[2] = {"pad.feats.0", "pad.feats.1"};
         if (src.kind == 2 && (padded || !tc_e4m3_supported(src.d) || (reinterpret_cast<uintptr_t>(src.feats) & 15)))
@@ -1518,7 +1519,7 @@ ludvig_status size_for_async(ludvig_scene* s, const std::vector<GroupViews>& gro
             n = std::max<int64_t>(g.nmax, 1);
         }
     }
-    return reserve_async(s, nv, ng, n, width, height, src, tc);
+    return reserve_async(s, nv, ng, n, width, height, src, tc, (int)std::min<size_t>(2, groups.size()));
 }
 
 // One uplift call: kind 0 adds into num/den, kind 1 zeroes them first and

@@ -131,10 +131,10 @@ ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int heig
 ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int NT, Arena& ws, int parity,
                          int* status, int64_t* chunk_cap, bool checked, cudaStream_t st, TileWeights* tw);
 
-// Allocates both buffer sets of the weight rows for groups of up to nitems
-// (view, tile) items and cap chunks (allocation synchronises the device, so an
-// asynchronous call that finds them in place never waits).
-ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap);
+// Allocates the first `sets` buffer sets of the weight rows for groups of up to
+// nitems (view, tile) items and cap chunks (allocation synchronises the device, so
+// an asynchronous call that finds them in place never waits).
+ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets);
 
 // num_v[i,:] += W^T F and den_v[i] += row sums for the group's weight rows
 // (k_aggregate_tc), view v's features at coordinate av.fview[v] of `feats`

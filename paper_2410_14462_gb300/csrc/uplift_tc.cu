@@ -1825,9 +1825,13 @@ const char* const kWsCounter[2] = {"tc.counter.0", "tc.counter.1"};
 const char* const kWsPlanOff[2] = {"tc.plan_off.0", "tc.plan_off.1"};
 const char* const kWsPlan[2] = {"tc.plan.0", "tc.plan.1"};
 
-ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap) {
-    cap = std::max<int64_t>(cap, 3 * (int64_t)nitems);
-    for (int p = 0; p < 2; ++p) {
+// Chunks a group's weight rows start with: three per tile (380 rows).  Float32
+// rows serve small images more often, whose tiles hold more Gaussians: four.
+int64_t start_chunks(int NT, int nitems) { return (NT == 3 ? 4 : 3) * (int64_t)nitems; }
+
+ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets) {
+    cap = std::max<int64_t>(cap, start_chunks(NT, nitems));
+    for (int p = 0; p < sets; ++p) {
         void* q;
         LV_TRY(ws.get(kWsCounter[p], sizeof(int), &q));
         LV_TRY(ws.get(kWsFirst[p], sizeof(int) * (size_t)nitems, &q));
@@ -1871,7 +1875,7 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         LV_TRY(ws.pinned("tc.host", 16, &hp));
         host = static_cast<int*>(hp);
     }
-    int64_t cap = std::max<int64_t>(*chunk_cap, 3 * (int64_t)nitems);
+    int64_t cap = std::max<int64_t>(*chunk_cap, start_chunks(NT, nitems));
     for (int attempt = 0; attempt < 2; ++attempt) {
         if (cap > 0x7fffffff / kCRows) {
             set_error("tile weights need %lld chunks of 128 rows", (long long)cap);

@@ -78,6 +78,17 @@ def test_cuda_core_features_not_finite():
     assert rel_l2(bad[~t].cpu().numpy(), out[~t].cpu().numpy()) <= 1e-5
 
 
+def test_fp8_cuda_core_width():
+    """Codes of a width the tensor cores do not take are decoded first."""
+    wl = inputs.small_field_workload(n=5000, views=2, d=36, width=61, height=45)
+    sc = ludvig.Scene.from_inputs(wl.scene)
+    q, s = ludvig.fp8_quantize(device_features(wl, range(2)))
+    x = (q.view(torch.float8_e4m3fn).float() * s.view(-1, 1, 1, 1)).bfloat16()
+    out, _ = ludvig.uplift_fp8(sc, wl.cams.params, 61, 45, q, s)
+    ref, _ = ludvig.uplift(sc, wl.cams.params, 61, 45, x.contiguous())
+    assert rel_l2(out.cpu().numpy(), ref.cpu().numpy()) <= 1e-6
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("elems", [1, 4096, 8192 + 5, 16384])
 def test_quantize_pieces(dtype, elems):
