@@ -512,8 +512,8 @@ ludvig_status ludvig_graph_destroy(ludvig_graph_t graph);
 /* Number of stored (directed) edges of the graph. Synchronises nothing. */
 int64_t ludvig_graph_nnz(ludvig_graph_t graph);
 
-/* Device bytes the graph's workspace holds now (diffusion scratch, the sliced
- * matrix copy); -1 for a NULL graph.  Same rules as
+/* Device bytes the graph's workspace holds now (diffusion scratch, the renumbered
+ * matrix copies); -1 for a NULL graph.  Same rules as
  * ludvig_scene_workspace_bytes. */
 int64_t ludvig_graph_workspace_bytes(ludvig_graph_t graph);
 
@@ -528,7 +528,8 @@ ludvig_status ludvig_graph_export(ludvig_graph_t graph, int64_t* row_ptr, int32_
  * 1 <= dx <= 32.  With dx = 1 the steps run on a sliced copy of the matrix
  * (32-row slices, column-major) that the first call after the graph's values
  * change builds in the graph's workspace; that call synchronises `stream`
- * once. */
+ * once.  More columns run on a renumbered row copy, built the same way (without
+ * a synchronisation). */
 ludvig_status ludvig_diffuse(ludvig_graph_t graph, const float* x0, int32_t dx, int32_t iters,
                              float* out, void* stream);
 

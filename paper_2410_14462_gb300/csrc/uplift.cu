@@ -636,7 +636,7 @@ struct RenderArgs {
 
 // CUDA-core rendering: one CTA per (view, tile) and DC channels (blockIdx.y),
 // one thread per pixel.  Walks the tile's list in batches of 32 Gaussians with
-// the compositing rules of k_composite and adds w f_i (the batch's DC-channel
+// the compositing rules of the walk (Eq. 1) and adds w f_i (the batch's DC-channel
 // feature slices staged in shared memory) into per-pixel registers in list
 // order; every pixel of the image is written (zero without contributors).
 template <int DC>
