@@ -160,6 +160,9 @@ struct ludvig_scene {
     // asynchronous uplift: front-end and aggregation streams, their events,
     // the device status words ([0] bounded-wait status, [1] capacity overflow)
     // and their host mirror with the groups' sizes
+    cudaStream_t st_pre = nullptr;        // the next group's projection and depth sort
+    cudaEvent_t ev_sorted = nullptr;      // on st_front: a group no longer reads what those write
+    cudaEvent_t ev_pre = nullptr;         // on st_pre: they are done
     cudaStream_t st_front = nullptr, st_agg = nullptr;
     cudaEvent_t ev_call = nullptr, ev_front[2] = {nullptr, nullptr}, ev_agg[2] = {nullptr, nullptr};
     cudaEvent_t ev_join[2] = {nullptr, nullptr}, ev_done = nullptr;
@@ -200,8 +203,9 @@ constexpr int kRadixTile = kRadixThreads * kRadixItems;   // keys per sort block
 // Exclusive prefix sum of n uint32 values (in-place allowed).  *total_dev
 // (device, may be null) receives the exact 64-bit sum; the uint32 prefixes are
 // meaningful only while that sum stays below 2^32.
+// side: scratch of its own, for a scan or sort that runs beside another of the same workspace.
 ludvig_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, uint64_t* total_dev,
-                                 Arena& ws, cudaStream_t st);
+                                 Arena& ws, cudaStream_t st, bool side = false);
 
 // Stable LSD radix sort of (key, value) pairs on key bits [0, nbits), applied
 // independently to nseg consecutive segments of seg_len entries each
@@ -209,7 +213,7 @@ ludvig_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, u
 // be swapped with (keys_alt, vals_alt).
 ludvig_status radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t* keys_alt,
                                uint32_t* vals_alt, int64_t nseg, int64_t seg_len, int nbits,
-                               Arena& ws, cudaStream_t st);
+                               Arena& ws, cudaStream_t st, bool side = false);
 
 // The same for one segment whose valid length is read on the device: `len`
 // (device, may be null = all of seg_len) entries of the seg_len-entry buffers

@@ -345,7 +345,7 @@ k_radix_downsweep(const KeyT* __restrict__ kin, const uint32_t* __restrict__ vin
 }  // namespace
 
 ludvig_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, uint64_t* total_dev,
-                                 Arena& ws, cudaStream_t st) {
+                                 Arena& ws, cudaStream_t st, bool side) {
     if (n <= 0) {
         if (total_dev) LV_CUDA(cudaMemsetAsync(total_dev, 0, sizeof(uint64_t), st));
         return LUDVIG_OK;
@@ -357,7 +357,7 @@ ludvig_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, u
     }
     const int64_t nb = ceil_div(n, kScanTile);
     unsigned long long* sums = nullptr;
-    LV_TRY(ws.get("scan.sums", (size_t)nb, &sums));
+    LV_TRY(ws.get(side ? "scan.sums.side" : "scan.sums", (size_t)nb, &sums));
     k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, sums);
     LV_LAUNCH();
     k_scan_sums<<<1, kScanThreads, 0, st>>>(sums, nb, reinterpret_cast<unsigned long long*>(total_dev));
@@ -367,16 +367,11 @@ ludvig_status scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, u
     return LUDVIG_OK;
 }
 
-ludvig_status radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t* keys_alt,
-                               uint32_t* vals_alt, int64_t nseg, int64_t seg_len, int nbits,
-                               Arena& ws, cudaStream_t st) {
-    return radix_sort_pairs_len(keys, vals, keys_alt, vals_alt, nseg, seg_len, nullptr, nbits, ws, st);
-}
-
 namespace {
 template <class KeyT>
 ludvig_status radix_sort_impl(KeyT** keys, uint32_t** vals, KeyT* keys_alt, uint32_t* vals_alt, int64_t nseg,
-                              int64_t seg_len, const uint64_t* len, int nbits, Arena& ws, cudaStream_t st) {
+                              int64_t seg_len, const uint64_t* len, int nbits, Arena& ws, cudaStream_t st,
+                              bool side = false) {
     if (len && nseg != 1) {
         set_error("radix_sort_pairs_len: a device length needs one segment");
         return LUDVIG_ERR_INTERNAL;
@@ -395,13 +390,13 @@ ludvig_status radix_sort_impl(KeyT** keys, uint32_t** vals, KeyT* keys_alt, uint
     }
     const int64_t nh = nseg * 256 * bps;
     uint32_t* hist = nullptr;
-    LV_TRY(ws.get("radix.hist", (size_t)nh, &hist));
+    LV_TRY(ws.get(side ? "radix.hist.side" : "radix.hist", (size_t)nh, &hist));
     KeyT *kin = *keys, *kout = keys_alt;
     uint32_t *vin = *vals, *vout = vals_alt;
     for (int shift = 0; shift < nbits; shift += 8) {
         k_radix_upsweep<KeyT><<<(unsigned)nblocks, kRadixThreads, 0, st>>>(kin, shift, hist, bps, len);
         LV_LAUNCH();
-        LV_TRY(scan_exclusive_u32(hist, hist, nh, nullptr, ws, st));
+        LV_TRY(scan_exclusive_u32(hist, hist, nh, nullptr, ws, st, side));
         k_radix_downsweep<KeyT><<<(unsigned)nblocks, kRadixThreads, 0, st>>>(kin, vin, kout, vout, shift,
                                                                              hist, bps, len);
         LV_LAUNCH();
@@ -417,6 +412,12 @@ ludvig_status radix_sort_impl(KeyT** keys, uint32_t** vals, KeyT* keys_alt, uint
     return LUDVIG_OK;
 }
 }  // namespace
+
+ludvig_status radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t* keys_alt,
+                               uint32_t* vals_alt, int64_t nseg, int64_t seg_len, int nbits,
+                               Arena& ws, cudaStream_t st, bool side) {
+    return radix_sort_impl<uint32_t>(keys, vals, keys_alt, vals_alt, nseg, seg_len, nullptr, nbits, ws, st, side);
+}
 
 ludvig_status radix_sort_pairs_len(uint32_t** keys, uint32_t** vals, uint32_t* keys_alt,
                                    uint32_t* vals_alt, int64_t nseg, int64_t seg_len, const uint64_t* len,

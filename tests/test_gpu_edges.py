@@ -51,6 +51,26 @@ def test_many_tiles(d, dtype, gate, count):
     assert _uplift_error(wl, dtype, count) <= gate
 
 
+# groups of 3, 3, 3 and 1 views whose depth sorts (74 tiles of keys a view) take the
+# several-block scan and run beside the group before; two calls, the second on a sized
+# workspace.  Sums of float32 in another order: the bar is the float32 uplift's.
+@pytest.mark.parametrize("d,dtype", [(3, torch.bfloat16), (40, torch.float32), (100, torch.float32)])
+def test_groups_sorted_ahead(d, dtype):
+    wl = inputs.small_field_workload(n=300_000, views=10, d=d, width=157, height=93)
+    sc = ludvig.Scene.from_inputs(wl.scene)
+    F = device_features(wl, range(10), dtype=dtype)
+    one, b1 = ludvig.uplift(sc, wl.cams.params, wl.cams.width, wl.cams.height, F)
+    saved = ludvig.get_option(ludvig.OPT_GROUP_MB)
+    ludvig.set_option(ludvig.OPT_GROUP_MB, 128)
+    try:
+        for _ in range(2):
+            many, bm = ludvig.uplift(sc, wl.cams.params, wl.cams.width, wl.cams.height, F)
+            assert rel_l2(many.cpu().numpy(), one.cpu().numpy()) <= 1e-5
+            assert rel_l2(bm.cpu().numpy(), b1.cpu().numpy()) <= 1e-5
+    finally:
+        ludvig.set_option(ludvig.OPT_GROUP_MB, saved)
+
+
 # weights of the CUDA-core path are float32, so bfloat16 features meet the float32 bar
 @pytest.mark.parametrize("d,dtype,count", [(33, torch.float32, False), (100, torch.float32, False),
                                            (101, torch.bfloat16, False), (132, torch.float32, True),
