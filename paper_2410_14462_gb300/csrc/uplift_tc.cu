@@ -109,7 +109,12 @@ struct WeightsArgs {
 
 constexpr int kDirectMaxD = 4;
 constexpr int kQuadItems = 152 * 16;
-constexpr int kBlockItems = 152 * 12;   // below: weight rows by blocks of 8 warps per tile
+// Below: weight rows by blocks of 8 warps per tile.  With few tiles the longest list
+// sets the time, and eight warps share it; from about 16 tiles an SM the warps of whole
+// tiles fill it.  Blocks against warps, uplifts of 64 channels, 300k clustered Gaussians:
+// 1920 tiles 864 and 937 us, 2349 tiles 1011 and 1203; 2660 tiles equal, 3600 tiles 1051
+// and 1008.  (Evenly spread scenes cross earlier: 1920 tiles 672 and 664, 2349 771 and 709.)
+constexpr int kBlockItems = 152 * 16;
 
 __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int rows, int next) {
     if (c >= 0 && c < a.cap) {
