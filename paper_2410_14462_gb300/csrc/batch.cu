@@ -15,7 +15,7 @@
 // that times candidate sizes on the class's own jobs the first time it meets
 // the class (LUDVIG_OPT_BATCH_TUNE), and kept for later batches.  The classes
 // run one after another, largest first, on one pooled context (a workspace,
-// two streams and their events) driven by the calling thread: each class
+// three streams and their events) driven by the calling thread: each class
 // fills the GPU with its groups, and one context bounds the weight-row
 // memory.
 //
