@@ -283,10 +283,10 @@ __device__ __forceinline__ float2 alpha_at_x2(F2 dx, F2 ax, F2 dy, F2 cy, F2 cb,
     const float ex = __uint_as_float((__float_as_uint(tt.x) << 23) + __float_as_uint(pp.x));
     const float ey = __uint_as_float((__float_as_uint(tt.y) << 23) + __float_as_uint(pp.y));
     const float2 al = f2_get(f2_mul(op, f2(ex, ey)));
-    const float a0 = fminf(al.x, kAlphaMax), a1 = fminf(al.y, kAlphaMax);
     const uint32_t lim = 0x42ae0000u;   // 87
-    return make_float2(__float_as_uint(mm.x) <= lim && a0 >= kAlphaMin ? a0 : 0.0f,
-                       __float_as_uint(mm.y) <= lim && a1 >= kAlphaMin ? a1 : 0.0f);
+    // the lower bound on alpha itself: a NaN (the opacity's) fails it, where fminf would make 0.99 of it
+    return make_float2(__float_as_uint(mm.x) <= lim && al.x >= kAlphaMin ? fminf(al.x, kAlphaMax) : 0.0f,
+                       __float_as_uint(mm.y) <= lim && al.y >= kAlphaMin ? fminf(al.y, kAlphaMax) : 0.0f);
 }
 
 // Conservative test: can a projected Gaussian reach alpha >= 1/255 at some
