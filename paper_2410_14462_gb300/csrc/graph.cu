@@ -183,8 +183,9 @@ __global__ void __launch_bounds__(128) k_knn(const float4* __restrict__ pts, int
                         if (ci == qi) continue;
                         const float ex = __fsub_rn(c.x, q.x), ey = __fsub_rn(c.y, q.y), ez = __fsub_rn(c.z, q.z);
                         const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
+                        // (a distance that is not a number, or overflowed, is no neighbour's)
                         const uint64_t key = ((uint64_t)__float_as_uint(d2) << 32) | ci;
-                        if (key < best[K - 1]) knn_insert(best, key);
+                        if (key < best[K - 1] && d2 <= FLT_MAX) knn_insert(best, key);
                     }
                 }
             }

@@ -51,3 +51,44 @@ def test_opacity_not_a_number_is_not_rendered():
     ref, got = (ludvig.render(ludvig.Scene.from_inputs(_with_opacity(wl.scene, bad, v)), wl.cams.params, 475, 269, f)
                 for v in (0.0, np.nan))
     assert rel_l2(got.cpu().numpy(), ref.cpu().numpy()) <= 1e-5
+
+
+def _scene_at(means):
+    n = len(means)
+    return inputs.Scene(means.astype(np.float32), np.full((n, 3), 0.01, np.float32),
+                        np.tile(np.array([1, 0, 0, 0], np.float32), (n, 1)), np.full(n, 0.5, np.float32))
+
+
+def _bad_centres(n):
+    """Clustered centres of which a few are not finite, or so far away that their squared distances overflow."""
+    means = inputs.scene_clusters(n, seed=4, n_clusters=6, sigma=0.1, extent=1.0).means.copy()
+    bad = np.array([0, 17, 500, n - 1])
+    means[0] = (np.nan, np.nan, np.nan)
+    means[17, 1] = np.nan
+    means[500] = 2e30
+    means[n - 1, 2] = np.nan
+    return means, bad, np.setdiff1d(np.arange(n), bad)
+
+
+@pytest.mark.parametrize("n,k", [(3000, 16), (20_000, 5), (1200, 40)])
+def test_centres_not_finite_have_no_neighbours(n, k):
+    means, bad, good = _bad_centres(n)
+    got = ludvig.knn(ludvig.Scene.from_inputs(_scene_at(means)), k).cpu().numpy()
+    ref = ludvig.knn(ludvig.Scene.from_inputs(_scene_at(means[good])), k).cpu().numpy()
+    assert (got[bad] == -1).all()
+    assert np.array_equal(got[good], good[ref])
+
+
+def test_centres_not_finite_leave_the_graph_alone():
+    n, k = 3000, 8
+    means, bad, good = _bad_centres(n)
+    f = np.random.default_rng(1).normal(size=(n, 24)).astype(np.float32)
+    x = np.random.default_rng(2).random((n, 3)).astype(np.float32)
+    x[bad] = 0.0
+    g = ludvig.Graph(ludvig.Scene.from_inputs(_scene_at(means)), k, torch.from_numpy(f).cuda(), spatial_h=0.01)
+    r = ludvig.Graph(ludvig.Scene.from_inputs(_scene_at(means[good])), k, torch.from_numpy(f[good]).cuda(), spatial_h=0.01)
+    for xs in (x, x[:, 0].copy()):
+        got = g.diffuse(torch.from_numpy(xs).cuda(), 5).cpu().numpy()
+        ref = r.diffuse(torch.from_numpy(xs[good]).cuda(), 5).cpu().numpy()
+        assert np.all(got[bad] == 0)
+        assert rel_l2(got[good], ref) <= 1e-5
