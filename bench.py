@@ -339,7 +339,7 @@ def roofline(tr, steps, alg_bytes_step, traffic_key=None, views_per_launch=None)
     (one per chunk of up to 16 views).  Time: CUDA events around each launch
     on the stream it runs on."""
     stage = "aggregate" if tr["calls"].get("aggregate", 0) > 0 else "composite"
-    kernel = "k_aggregate_tc" if stage == "aggregate" else "k_aggregate_cc"
+    kernel = "k_aggregate_tc" if stage == "aggregate" else "k_composite"
     launch_ms = tr["ms"][stage] / max(1, tr["calls"][stage])
     launches = tr["calls"][stage] / steps
     alg_per_launch = alg_bytes_step / max(1.0, launches)

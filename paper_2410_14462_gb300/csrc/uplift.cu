@@ -14,11 +14,11 @@
 //                  tile's list stays in (depth, index) order
 //   5. ranges      [start, end) of every (view, tile) list
 //   6. weights + aggregate (uplift_tc.cu): the weight rows of every tile,
-//                  gathering the walked records by rank, then W^T F.  For d <= 4
-//                  the walk adds its sums itself; for d < 32 (features zero-padded
-//                  to 32 channels) and 32 <= d <= 512 with d % 8 == 0 the product
-//                  runs on the tensor cores (tcgen05) on bfloat16 terms; otherwise
-//                  here on CUDA cores on float32 rows (k_aggregate_cc).
+//                  gathering the walked records by rank, then W^T F on the
+//                  tensor cores (tcgen05), for d < 32 (features zero-padded to
+//                  32 channels; for d <= 4 the walk adds its sums itself) and
+//                  for 32 <= d <= 512 with d % 8 == 0; otherwise here on CUDA
+//                  cores (k_composite), walk and product in one kernel.
 //   7. normalise   f = num / den (den > 0), beta = den.
 //
 // The uplift entry points do not wait on the host.  The pair count and the
@@ -390,8 +390,11 @@ __global__ void k_pair_records(const uint32_t* __restrict__ pkey, const uint32_t
     }
 }
 
-// ------------------------------------------------------------ 6. aggregate on CUDA cores
-constexpr int kBatch = 32;        // Gaussians composited per step (k_render_cc, k_transmittance)
+// ------------------------------------------------------------ 6. composite + aggregate
+constexpr int kBatch = 32;        // Gaussians composited per step
+constexpr int kStoreCap = 12288;  // non-zero weights kept per flush
+constexpr int kRowCap = 1024;     // Gaussians kept per flush
+constexpr int kChunk = 32;        // channels per aggregation chunk (vector path)
 
 __device__ __forceinline__ void red_add_v4(float* addr, float4 v) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(v.x), "f"(v.y),
@@ -402,225 +405,245 @@ __device__ __forceinline__ void red_add_v4(float* addr, float4 v) {
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 
-__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
-    const uint2 q = *reinterpret_cast<const uint2*>(p);
-    return make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u), __uint_as_float(q.y << 16),
-                       __uint_as_float(q.y & 0xffff0000u));
+struct CompositeArgs {
+    const PairRec* pairs;   // list records in list order
+    const uint2* ranges;
+    int ntiles, TX, width, height;
+    const void* feats;      // chunk's first view
+    int d;
+    float* num;
+    float* den;
+    float* dbg_t;           // [H*W] view 0 only, or null
+    int32_t* dbg_cnt;
+    int count_den;          // den += the number of non-zero weights instead of their sum
+};
+
+struct CompositeSmem {
+    float4 ra[kBatch];
+    float2 rb[kBatch];
+    uint32_t gid[kBatch];
+    uint32_t bmask[kBatch];
+    uint32_t wcnt[8][kBatch];
+    uint32_t rtot[kBatch];
+    uint32_t rbase[kBatch];
+    uint32_t row_gid[kRowCap];
+    uint32_t row_start[kRowCap];
+    uint32_t row_cnt[kRowCap];
+    float store_w[kStoreCap];
+    uint8_t store_p[kStoreCap];
+    int nstore, nrows;
+    alignas(16) float F[256 * kChunk];
+};
+
+template <class TIn, bool kVec>
+__device__ void flush_store(CompositeSmem& sm, const CompositeArgs& a, const TIn* __restrict__ fv,
+                            int tx, int ty) {
+    __syncthreads();
+    const int R = sm.nrows;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (R > 0) {
+        // beta_i partial: sum of the Gaussian's stored weights
+        for (int r = warp; r < R; r += 8) {
+            const uint32_t st = sm.row_start[r], c = sm.row_cnt[r];
+            float s = 0.f;
+            for (uint32_t k = lane; k < c; k += 32) s += a.count_den ? 1.f : sm.store_w[st + k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) atomicAdd(a.den + sm.row_gid[r], s);
+        }
+        const int d = a.d;
+        constexpr int cw = kVec ? kChunk : 8;   // channels per chunk
+        for (int c0 = 0; c0 < d; c0 += cw) {
+            const int dcw = min(cw, d - c0);
+            // stage F[tile pixels][c0 : c0+dcw) (zeros outside the image)
+            for (int idx = tid; idx < 256 * cw; idx += 256) {
+                const int p = idx / cw, c = idx % cw;
+                const int px = tx * kTile + (p & 15), py = ty * kTile + (p >> 4);
+                float val = 0.f;
+                if (c < dcw && px < a.width && py < a.height)
+                    val = to_f32(fv[((int64_t)py * a.width + px) * d + c0 + c]);
+                sm.F[p * kChunk + c] = val;
+            }
+            __syncthreads();
+            if (kVec) {
+                const int q = lane & 7;
+                for (int r = warp * 4 + (lane >> 3); r < R; r += 32) {
+                    const uint32_t st = sm.row_start[r], c = sm.row_cnt[r];
+                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (uint32_t k = 0; k < c; ++k) {
+                        const int p = sm.store_p[st + k];
+                        const float w = sm.store_w[st + k];
+                        const float4 f = *reinterpret_cast<const float4*>(&sm.F[p * kChunk + 4 * q]);
+                        acc.x = fmaf(w, f.x, acc.x);
+                        acc.y = fmaf(w, f.y, acc.y);
+                        acc.z = fmaf(w, f.z, acc.z);
+                        acc.w = fmaf(w, f.w, acc.w);
+                    }
+                    if (4 * q < dcw) red_add_v4(a.num + (int64_t)sm.row_gid[r] * d + c0 + 4 * q, acc);
+                }
+            } else {
+                const int q = lane & 7;
+                for (int r = warp * 4 + (lane >> 3); r < R; r += 32) {
+                    const uint32_t st = sm.row_start[r], c = sm.row_cnt[r];
+                    float acc = 0.f;
+                    for (uint32_t k = 0; k < c; ++k)
+                        acc = fmaf(sm.store_w[st + k], sm.F[sm.store_p[st + k] * kChunk + q], acc);
+                    if (q < dcw) atomicAdd(a.num + (int64_t)sm.row_gid[r] * d + c0 + q, acc);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (threadIdx.x == 0) {
+        sm.nstore = 0;
+        sm.nrows = 0;
+    }
+    __syncthreads();
 }
 
-// num[i, :] += sum_p w_i(p) F[p, :] over a tile's float32 weight rows, for the
-// widths (and the option) the tensor cores do not take.
-struct CcArgs {
-    const float* w;             // [cap][128][256] float32 weight rows
-    const uint32_t* chunk_gid;
-    const float* chunk_den;     // [cap][128]
-    const uint32_t* plan_off;   // the item's chunks: plan[plan_off[item] ..)
-    const int2* plan;
-    const int* chunk_count;     // chunks the weights pass used (null: known to fit)
-    int cap;
-    int* ovf;                   // set to 2 when they exceeded cap (nothing is added)
-    int ntiles, TX, width, height, d, nblk;
-    int vec4;                   // num rows take 16-byte reductions
-    int vecf;                   // four channels of a pixel are one aligned load
-    const void* feats;          // [.., H, W, d], views at views.fview
-    AggViews views;
-};
-
-// A block of 128 threads takes 128 channels of a (view, tile), its rows 64 at a
-// time, as a dense product over the tile's 256 pixels in eight steps of 32: the
-// step's 64 rows x 32 pixels and 32 pixels x 128 channels are staged in shared
-// memory (the next step's loads in flight behind the current one), a thread
-// multiplies 8 rows x 8 channels (smaller tiles are bound by their shared-memory
-// reads: 4 x 4 took twice the time).  A weight of zero must not meet an infinite
-// or NaN feature, so a step whose features are not all finite skips zero weights.
-// Bound: the FMA pipe (rows rounded up to 64, channels to 128).  About 40 % of a
-// row's weights are non-zero, but a sparse store of them cost three shared-memory
-// loads per four multiply-adds: 10 views of 331x227 with 100 float32 channels took
-// 2.97 ms in one kernel with its walk, now 1.85 (0.56 of the pipe) + 0.60.
-constexpr int kCcPx = 32;                      // pixels per step
-constexpr int kCcWPitch = kCcPx + 4, kCcFPitch = 128 + 4;   // floats per staged line (16-byte aligned)
-
-struct CcSmem {
-    float w[2][64 * kCcWPitch];      // [row][pixel]
-    float f[2][kCcPx * kCcFPitch];   // [pixel][channel]
-};
-
-template <class TIn>
-__global__ void __launch_bounds__(128, 3) k_aggregate_cc(const __grid_constant__ CcArgs a) {
+// One CTA (256 threads = 16x16 pixels) per (view, tile), over list records with
+// their 8x4 block masks: walks the list in batches of 32 Gaussians, forms
+// w = alpha T per pixel, keeps the tile's non-zero weights in a shared-memory sparse
+// store grouped by Gaussian, then multiplies the store with the tile's feature rows
+// (staged by channel chunks) and adds every Gaussian's partial sum into num / den
+// with vector reductions.  Bound by the product's shared-memory reads (three per
+// four multiply-adds).
+// Float32 weight rows in global memory and a dense product on register tiles take
+// less time on a sized workspace (10 views of 331x227, 100 float32 channels: 3.39 ms
+// here, 2.91 with rows; 8 views of 640x480 7.16 and 3.82), but half a megabyte of rows a
+// tile: a scene's first call took longer (4.5 and 5.8 ms; 8.4 and 9.4, with 0.3 and
+// 7.4 GB held), and so did calls of few tiles (80 tiles 1.27 and 1.81 ms, 300 0.93 and
+// 1.12).
+template <class TIn, bool kVec>
+__global__ void __launch_bounds__(256, 2) k_composite(CompositeArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    CcSmem& S = *reinterpret_cast<CcSmem*>(smem_raw);
-    if (a.chunk_count && *a.chunk_count > a.cap) {   // incomplete rows: the group is redone
-        if (blockIdx.x == 0 && threadIdx.x == 0 && a.ovf) atomicOr(a.ovf, 2);
-        return;
-    }
-    const int item = (int)(blockIdx.x / (unsigned)a.nblk), blk = (int)(blockIdx.x - (unsigned)item * (unsigned)a.nblk);
-    const uint32_t k0 = a.plan_off[item], k1 = a.plan_off[item + 1];
-    if (k0 >= k1) return;
+    CompositeSmem& sm = *reinterpret_cast<CompositeSmem*>(smem_raw);
+    const int item = blockIdx.x;
     const int v = item / a.ntiles, tile = item - v * a.ntiles;
     const int tx = tile % a.TX, ty = tile / a.TX;
-    const int d = a.d, c0 = 128 * blk, dc = min(128, d - c0);
-    // thread: rows rg, rg + 8 .. (the two rows a warp reads lie four banks apart),
-    // channels 4 cg .. + 3 and 64 + 4 cg .. + 3
-    const int tid = threadIdx.x, cg = tid & 15, rg = tid >> 4;
-    const TIn* fv = static_cast<const TIn*>(a.feats) + (size_t)a.views.fview[v] * a.height * a.width * d + c0;
-    float* const num = a.views.num[v];
-    float* const den = a.views.den[v];
-    // features of a step: channels 4 (tid & 31) .. + 3 of pixels (tid >> 5) + 4 e
-    constexpr int kF = kCcPx / 4;
-    float4 fr[kF];
-    auto load_f = [&](int ka) {
-        const int ch = 4 * (tid & 31);
-#pragma unroll
-        for (int e = 0; e < kF; ++e) {
-            const int p = kCcPx * ka + (tid >> 5) + 4 * e, px = tx * kTile + (p & 15), py = ty * kTile + (p >> 4);
-            fr[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (px >= a.width || py >= a.height) continue;
-            const TIn* src = fv + ((size_t)py * a.width + px) * d + ch;
-            if (a.vecf) {   // (dc is a multiple of 4)
-                if (ch < dc) fr[e] = load4(src);
-            } else {
-                if (ch < dc) fr[e].x = to_f32(src[0]);
-                if (ch + 1 < dc) fr[e].y = to_f32(src[1]);
-                if (ch + 2 < dc) fr[e].z = to_f32(src[2]);
-                if (ch + 3 < dc) fr[e].w = to_f32(src[3]);
-            }
-        }
-    };
-    for (uint32_t k = k0; k < k1; ++k) {
-        const int2 pl = a.plan[k];
-        for (int rb = 0; rb < pl.y; rb += 64) {
-            const int nr = min(64, pl.y - rb);
-            const float* wrow = a.w + ((size_t)pl.x * 128 + rb) * 256;
-            auto load_w = [&](int ka, int buf) {   // 16 bytes x 4 per thread: rows (tid >> 3) + 16 e
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int row = (tid >> 3) + 16 * e, p = 4 * (tid & 7);
-                    if (row < nr) {
-                        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&S.w[buf][row * kCcWPitch + p]);
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                                     "l"(wrow + (size_t)row * 256 + kCcPx * ka + p)
-                                     : "memory");
-                    }
-                }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-            };
-            float acc[8][8];
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-            __syncthreads();   // the previous rows' stages are used up
-            load_w(0, 0);
-            load_f(0);
-            for (int ka = 0; ka < 256 / kCcPx; ++ka) {
-                const int buf = ka & 1;
-                bool odd = false;
-#pragma unroll
-                for (int e = 0; e < kF; ++e) {
-                    *reinterpret_cast<float4*>(&S.f[buf][((tid >> 5) + 4 * e) * kCcFPitch + 4 * (tid & 31)]) = fr[e];
-                    odd |= !(isfinite(fr[e].x) && isfinite(fr[e].y) && isfinite(fr[e].z) && isfinite(fr[e].w));
-                }
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                const int any_odd = __syncthreads_or(odd);
-                if (ka + 1 < 256 / kCcPx) {   // the other stage was used up before the barrier
-                    load_w(ka + 1, buf ^ 1);
-                    load_f(ka + 1);
-                }
-                const float* ws = &S.w[buf][rg * kCcWPitch];
-                const float* fp = &S.f[buf][4 * cg];
-                auto step = [&](auto guard) {
-#pragma unroll 2
-                    for (int p = 0; p < kCcPx; p += 4) {
-                        float4 w[8];
-#pragma unroll
-                        for (int r = 0; r < 8; ++r) w[r] = *reinterpret_cast<const float4*>(ws + 8 * r * kCcWPitch + p);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float4 f0 = *reinterpret_cast<const float4*>(fp + (p + q) * kCcFPitch);
-                            const float4 f1 = *reinterpret_cast<const float4*>(fp + (p + q) * kCcFPitch + 64);
-#pragma unroll
-                            for (int r = 0; r < 8; ++r) {
-                                const float x = q == 0 ? w[r].x : q == 1 ? w[r].y : q == 2 ? w[r].z : w[r].w;
-                                if (guard.value && x == 0.f) continue;
-                                acc[r][0] = fmaf(x, f0.x, acc[r][0]);
-                                acc[r][1] = fmaf(x, f0.y, acc[r][1]);
-                                acc[r][2] = fmaf(x, f0.z, acc[r][2]);
-                                acc[r][3] = fmaf(x, f0.w, acc[r][3]);
-                                acc[r][4] = fmaf(x, f1.x, acc[r][4]);
-                                acc[r][5] = fmaf(x, f1.y, acc[r][5]);
-                                acc[r][6] = fmaf(x, f1.z, acc[r][6]);
-                                acc[r][7] = fmaf(x, f1.w, acc[r][7]);
-                            }
-                        }
-                    }
-                };
-                if (any_odd)
-                    step(std::true_type{});
-                else
-                    step(std::false_type{});
-            }
-#pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                const int row = rg + 8 * r;
-                if (row >= nr) continue;
-                const size_t slot = (size_t)pl.x * 128 + rb + row;
-                const uint32_t g = a.chunk_gid[slot];
-                if (blk == 0 && cg == 0) atomicAdd(den + g, a.chunk_den[slot]);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int ch = 64 * h + 4 * cg;
-                    if (ch >= dc) continue;
-                    float* dst = num + (size_t)g * d + c0 + ch;
-                    if (a.vec4) {
-                        red_add_v4(dst, make_float4(acc[r][4 * h], acc[r][4 * h + 1], acc[r][4 * h + 2],
-                                                    acc[r][4 * h + 3]));
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (ch + c < dc) atomicAdd(dst + c, acc[r][4 * h + c]);
-                    }
-                }
-            }
-        }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    // warp w covers the 8x4 pixel block ((w & 1) * 8, (w >> 1) * 4) of the tile
+    const int bx = (warp & 1) * 8, by = (warp >> 1) * 4;
+    const int lx = bx + (lane & 7), ly = by + (lane >> 3);
+    const int pix = ly * kTile + lx;   // tile-local pixel index
+    const int px = tx * kTile + lx, py = ty * kTile + ly;
+    const bool inside = px < a.width && py < a.height;
+    const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
+    const uint2 range = a.ranges[item];
+    const TIn* fv = reinterpret_cast<const TIn*>(a.feats) + (int64_t)v * a.height * a.width * a.d;
+    if (tid == 0) {
+        sm.nstore = 0;
+        sm.nrows = 0;
     }
-}
-
-// The walk alone, for inspection: every pixel's transmittance after it and its
-// number of contributors (one block of 256 threads per tile of one view).
-__global__ void __launch_bounds__(256) k_transmittance(const PairRec* __restrict__ pairs,
-                                                       const uint2* __restrict__ ranges, int TX, int width, int height,
-                                                       float* __restrict__ t_final, int32_t* __restrict__ n_contrib) {
-    __shared__ PairRec rec[kBatch];
-    const int tx = (int)blockIdx.x % TX, ty = (int)blockIdx.x / TX, tid = threadIdx.x;
-    const int px = tx * kTile + (tid & 15), py = ty * kTile + (tid >> 4);
-    const bool inside = px < width && py < height;
-    const uint2 range = ranges[blockIdx.x];
+    // records of the next batch, loaded one batch ahead
+    PairRec nxt{};
+    if (tid < kBatch && range.x + tid < range.y) nxt = a.pairs[range.x + tid];
     float T = 1.0f;
     bool done = !inside;
-    int cnt = 0;
+    int ncontrib = 0;
+    __syncthreads();
     for (uint32_t b0 = range.x; b0 < range.y; b0 += kBatch) {
         if (__syncthreads_count(!done) == 0) break;
-        const int nb = (int)min((uint32_t)kBatch, range.y - b0);
-        if (tid < nb) rec[tid] = pairs[b0 + tid];
+        const int cnt = (int)min((uint32_t)kBatch, range.y - b0);
+        if (sm.nstore + kBatch * 256 > kStoreCap || sm.nrows + kBatch > kRowCap)
+            flush_store<TIn, kVec>(sm, a, fv, tx, ty);
+        if (tid < cnt) {
+            sm.gid[tid] = nxt.gid;
+            sm.bmask[tid] = nxt.mask;
+            sm.ra[tid] = make_float4(nxt.mx, nxt.my, nxt.ca, nxt.cb);
+            sm.rb[tid] = make_float2(nxt.cc, nxt.op);
+        }
+        if (tid < kBatch && b0 + kBatch + tid < range.y) nxt = a.pairs[b0 + kBatch + tid];
         __syncthreads();
-        for (int j = 0; j < nb && !done; ++j) {
-            const PairRec& r = rec[j];
-            const float al = alpha_at(r.mx, r.my, r.ca, r.cb, r.cc, r.op, (float)px + 0.5f, (float)py + 0.5f);
-            if (al > 0.f) {
+        // Gaussians of the batch that can reach this warp's pixel block
+        uint32_t rel = __ballot_sync(0xffffffffu, lane < cnt && ((sm.bmask[lane] >> warp) & 1u));
+        if (!__any_sync(0xffffffffu, !done)) rel = 0u;
+        // alphas of the batch first (independent chains the scheduler can
+        // overlap), then the sequential transmittance recursion
+        float w[kBatch];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            w[j] = 0.f;
+            if ((rel >> j) & 1u) {
+                const float4 ra = sm.ra[j];
+                const float2 rb = sm.rb[j];
+                w[j] = alpha_at(ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, pxf, pyf);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const float al = w[j];
+            w[j] = 0.f;
+            if (al > 0.f && !done) {
                 const float Tn = __fmul_rn(T, __fsub_rn(1.0f, al));
                 if (Tn < kTransMin) {
                     done = true;
                 } else {
+                    w[j] = __fmul_rn(al, T);
                     T = Tn;
-                    ++cnt;
+                    ++ncontrib;
                 }
             }
         }
+        // per-warp counts of non-zero weights of every Gaussian of the batch
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const uint32_t m = __ballot_sync(0xffffffffu, w[j] != 0.f);
+            if (lane == 0) sm.wcnt[warp][j] = __popc(m);
+        }
+        __syncthreads();
+        if (tid < kBatch) {
+            uint32_t t = 0;
+#pragma unroll
+            for (int wi = 0; wi < 8; ++wi) {
+                const uint32_t c = sm.wcnt[wi][tid];
+                sm.wcnt[wi][tid] = t;
+                t += c;
+            }
+            sm.rtot[tid] = t;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const int ns = sm.nstore, nr = sm.nrows;
+            const uint32_t t = lane < cnt ? sm.rtot[lane] : 0u;
+            uint32_t incl = t;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            const uint32_t start = (uint32_t)ns + incl - t;
+            sm.rbase[lane] = start;
+            const uint32_t nzm = __ballot_sync(0xffffffffu, t > 0);
+            if (t > 0) {
+                const int slot = nr + __popc(nzm & lt_mask);
+                sm.row_gid[slot] = sm.gid[lane];
+                sm.row_start[slot] = start;
+                sm.row_cnt[slot] = t;
+            }
+            __syncwarp();
+            if (lane == 31) {
+                sm.nstore = ns + (int)incl;
+                sm.nrows = nr + __popc(nzm);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const uint32_t m = __ballot_sync(0xffffffffu, w[j] != 0.f);
+            if (w[j] != 0.f) {
+                const uint32_t pos = sm.rbase[j] + sm.wcnt[warp][j] + __popc(m & lt_mask);
+                sm.store_w[pos] = w[j];
+                sm.store_p[pos] = (uint8_t)pix;
+            }
+        }
+        __syncthreads();
     }
-    if (inside) {
-        t_final[(int64_t)py * width + px] = T;
-        n_contrib[(int64_t)py * width + px] = cnt;
+    flush_store<TIn, kVec>(sm, a, fv, tx, ty);
+    if (a.dbg_t && v == 0 && inside) {
+        a.dbg_t[(int64_t)py * a.width + px] = T;
+        a.dbg_cnt[(int64_t)py * a.width + px] = ncontrib;
     }
 }
 
@@ -636,7 +659,7 @@ struct RenderArgs {
 
 // CUDA-core rendering: one CTA per (view, tile) and DC channels (blockIdx.y),
 // one thread per pixel.  Walks the tile's list in batches of 32 Gaussians with
-// the compositing rules of the walk (Eq. 1) and adds w f_i (the batch's DC-channel
+// the compositing rules of k_composite and adds w f_i (the batch's DC-channel
 // feature slices staged in shared memory) into per-pixel registers in list
 // order; every pixel of the image is written (zero without contributors).
 template <int DC>
@@ -777,6 +800,8 @@ struct ChunkDebug {
     int64_t* list_total = nullptr;  // host
     bool stop_after_sort = false;
     bool unpruned = false;          // lists by the tile-rectangle rule alone
+    float* t_final = nullptr;
+    int32_t* n_contrib = nullptr;
 };
 
 __global__ void k_export_ranges(const uint2* __restrict__ r, int64_t nt, int64_t* __restrict__ out) {
@@ -801,6 +826,19 @@ __global__ void k_export_list(const uint32_t* __restrict__ pkey, const uint32_t*
     if (j >= P) return;
     const int64_t v = pkey[j] / (uint32_t)ntiles;
     out[j] = (int32_t)srec[v * npad + pval[j]].gid;
+}
+
+size_t composite_smem() { return sizeof(CompositeSmem); }
+
+template <class TIn, bool kVec>
+ludvig_status launch_composite(const CompositeArgs& args, int64_t nitems, cudaStream_t st) {
+    // set once per process; a function-local static is initialised by one thread
+    static const cudaError_t configured =
+        cudaFuncSetAttribute(k_composite<TIn, kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)composite_smem());
+    LV_CUDA(configured);
+    k_composite<TIn, kVec><<<(unsigned)nitems, 256, composite_smem(), st>>>(args);
+    LV_LAUNCH();
+    return LUDVIG_OK;
 }
 
 template <int DC>
@@ -1095,51 +1133,40 @@ ludvig_status front_end(ludvig_scene* ctx, const GroupViews& g, int width, int h
     return LUDVIG_OK;
 }
 
-// CUDA-core aggregation of a group's float32 weight rows (k_aggregate_cc).
-template <class TIn>
-ludvig_status launch_cc(const CcArgs& args, unsigned grid, cudaStream_t st) {
-    // set once per process; a function-local static is initialised by one thread
-    static const cudaError_t configured =
-        cudaFuncSetAttribute(k_aggregate_cc<TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CcSmem));
-    LV_CUDA(configured);
-    k_aggregate_cc<TIn><<<grid, 128, sizeof(CcSmem), st>>>(args);
-    LV_LAUNCH();
-    return LUDVIG_OK;
-}
-
-ludvig_status aggregate_cc(const TileWeights& t, int nv, int width, int height, const void* feats, int dtype, int d,
-                           const AggViews& av, int* ovf, cudaStream_t st) {
+// CUDA-core stage 6 of a group (k_composite): the list records with their
+// block masks, then the per-tile composite with its shared-memory weight store.
+ludvig_status composite_cc(ludvig_scene* s, const FrontEnd& fe, int nv, int width, int height, const void* feats,
+                           int dtype, int d, float* num, float* den, const ChunkDebug* dbg, cudaStream_t st) {
     const int TX = (width + kTile - 1) / kTile, TY = (height + kTile - 1) / kTile;
-    const int64_t nitems = (int64_t)nv * TX * TY;
-    if (nitems == 0 || t.count == 0) return LUDVIG_OK;
-    CcArgs a{};
-    a.w = reinterpret_cast<const float*>(t.wg1);
-    a.chunk_gid = t.cgid;
-    a.chunk_den = t.cden;
-    a.plan_off = t.plan_off;
-    a.plan = t.plan;
-    a.chunk_count = t.count >= 0 ? nullptr : t.counter;   // a checked run already fits
-    a.cap = (int)t.cap;
-    a.ovf = ovf;
-    a.ntiles = TX * TY;
-    a.TX = TX;
-    a.width = width;
-    a.height = height;
-    a.d = d;
-    a.nblk = (d + 127) / 128;
-    a.feats = feats;
-    a.views = av;
-    a.vec4 = d % 4 == 0 ? 1 : 0;
-    a.vecf = d % 4 == 0 && reinterpret_cast<uintptr_t>(feats) % (dtype == LUDVIG_F32 ? 16 : 8) == 0 ? 1 : 0;
-    for (int k = 0; k < nv; ++k)
-        if (reinterpret_cast<uintptr_t>(av.num[k]) & 15) a.vec4 = 0;
-    if (nitems * a.nblk > 0x7fffffff) {
-        set_error("too many tiles for %d channels in one group", d);
-        return LUDVIG_ERR_INTERNAL;
-    }
+    const int ntiles = TX * TY;
+    PairRec* pairs;
+    LV_TRY(s->ws.get("up.pairs", (size_t)fe.cap, &pairs));
     StageScope scope(LUDVIG_STAGE_COMPOSITE, st);
-    const unsigned grid = (unsigned)(nitems * a.nblk);
-    return dtype == LUDVIG_F32 ? launch_cc<float>(a, grid, st) : launch_cc<__nv_bfloat16>(a, grid, st);
+    k_pair_records<<<kPairGrid, 256, 0, st>>>(fe.spk, fe.L.rank, fe.np, (uint64_t)fe.cap, ntiles, TX, fe.L.npad,
+                                              fe.L.srec, pairs);
+    LV_LAUNCH();
+    CompositeArgs args;
+    args.pairs = pairs;
+    args.ranges = fe.L.ranges;
+    args.ntiles = ntiles;
+    args.TX = TX;
+    args.width = width;
+    args.height = height;
+    args.feats = feats;
+    args.d = d;
+    args.num = num;
+    args.den = den;
+    args.dbg_t = dbg ? dbg->t_final : nullptr;
+    args.dbg_cnt = dbg ? dbg->n_contrib : nullptr;
+    args.count_den = option_count_normalise() ? 1 : 0;
+    const int64_t nitems = (int64_t)nv * ntiles;
+    const bool vec = (d % 4 == 0);
+    if (dtype == LUDVIG_F32) {
+        if (vec) return launch_composite<float, true>(args, nitems, st);
+        return launch_composite<float, false>(args, nitems, st);
+    }
+    if (vec) return launch_composite<__nv_bfloat16, true>(args, nitems, st);
+    return launch_composite<__nv_bfloat16, false>(args, nitems, st);
 }
 
 // ---------------------------------------------------------------- group pipeline
@@ -1181,7 +1208,7 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
     }
     FrontEnd fe;
     if (ex.presorted) LV_CUDA(cudaStreamWaitEvent(sf, s->ev_pre, 0));
-    LV_TRY(front_end(s, g, width, height, !ex.async, ex.async ? ex.ovf : nullptr, nullptr, sf, &fe, true,
+    LV_TRY(front_end(s, g, width, height, !ex.async, ex.async ? ex.ovf : nullptr, nullptr, sf, &fe, tc,
                      ex.presorted));
     if (ex.async) LV_CUDA(cudaEventRecord(s->ev_sorted, sf));
     if (fe.too_many) {
@@ -1190,7 +1217,7 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
     }
     if (ex.async) LV_CUDA(cudaMemcpyAsync(&ex.diag->pairs, fe.np, sizeof(uint64_t), cudaMemcpyDeviceToDevice, sf));
     if (pair_cap) *pair_cap = fe.cap;
-    if (chunk_cap) *chunk_cap = 0x7fffffff;   // no weight rows where the walk accumulates itself
+    if (chunk_cap) *chunk_cap = 0x7fffffff;   // no weight rows on CUDA cores or where the walk accumulates itself
     const int64_t view_elems = (int64_t)width * height * src.d;
     const size_t esize = src.kind == 2 ? 1 : (src.dtype == LUDVIG_F32 ? 4 : 2);
     const int fv0 = g.v[0].fview;
@@ -1199,9 +1226,9 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
     // a one-scene group's features start at its first coordinate
     const void* f0 = static_cast<const char*>(src.feats) + (size_t)fv0 * view_elems * esize;
 
-    // the operand features and the weight rows go to the buffer set of parity
-    // p, free once the aggregation of group - 2 is done
-    if (ex.async && ex.group >= 2) LV_CUDA(cudaStreamWaitEvent(sf, s->ev_agg[p], 0));
+    // the operand features and the weight rows of the tensor cores go to the
+    // buffer set of parity p, free once the aggregation of group - 2 is done
+    if (tc && ex.async && ex.group >= 2) LV_CUDA(cudaStreamWaitEvent(sf, s->ev_agg[p], 0));
     static const char* const kFb[2] = {"fp8.bf16.0", "fp8.bf16.1"};
     static const char* const kPad[2] = {"pad.feats.0", "pad.feats.1"};
     AggViews av;
@@ -1230,6 +1257,9 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
         fextent = nv;
         for (int k = 0; k < nv; ++k) av.fview[k] = k;
     }
+    if (!tc)
+        return composite_cc(s, fe, nv, width, height, src.kind == 2 ? f : f0, fdt, deff, g.v[0].num, g.v[0].den,
+                            nullptr, sf);
     if (src_direct(src)) {
         // a few channels: the weights pass adds each row's W^T F and den into
         // the (padded) numerator itself; no weight rows, no aggregation
@@ -1266,7 +1296,7 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
         for (int k = 0; k < nv; ++k) av.fview[k] = k;
     }
     TileWeights t;
-    LV_TRY(tc_weights(fe.L, nv, width, height, !tc ? 3 : fdt == LUDVIG_F32 ? 2 : 1, s->ws, p, s->dstat,
+    LV_TRY(tc_weights(fe.L, nv, width, height, fdt == LUDVIG_F32 ? 2 : 1, s->ws, p, s->dstat,
                       &s->tc_chunk_cap, !ex.async, sf, &t));
     if (chunk_cap) *chunk_cap = t.cap;
     if (ex.async) {
@@ -1274,11 +1304,8 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
         LV_CUDA(cudaEventRecord(s->ev_front[p], sf));
         LV_CUDA(cudaStreamWaitEvent(sa, s->ev_front[p], 0));
     }
-    if (!tc)
-        LV_TRY(aggregate_cc(t, nv, width, height, f, fdt, deff, av, ex.async ? ex.ovf : nullptr, sa));
-    else
-        LV_TRY(tc_aggregate(t, nv, width, height, f, fextent, f8_in_kernel ? kDtypeE4M3 : fdt, deff, av, s->dstat,
-                            ex.async ? ex.ovf : nullptr, sa, f8_in_kernel ? src.scales : nullptr));
+    LV_TRY(tc_aggregate(t, nv, width, height, f, fextent, f8_in_kernel ? kDtypeE4M3 : fdt, deff, av, s->dstat,
+                        ex.async ? ex.ovf : nullptr, sa, f8_in_kernel ? src.scales : nullptr));
     if (ex.async) LV_CUDA(cudaEventRecord(s->ev_agg[p], sa));
     return LUDVIG_OK;
 }
@@ -1363,7 +1390,10 @@ ludvig_status reserve_async(ludvig_scene* s, int nv, int ng, int64_t n, int widt
     const bool padded = src_padded(src);
     const int fdt = src.kind == 2 ? LUDVIG_BF16 : src.dtype;
     const bool direct = src_direct(src);   // no weight rows, no padded copy
-    if (!direct) LV_TRY(tc_reserve(ws, !tc ? 3 : fdt == LUDVIG_F32 ? 2 : 1, nv * TX * TY, s->tc_chunk_cap, sets));
+    if (!tc)
+        LV_TRY(ws.get("up.pairs", sizeof(PairRec) * (size_t)cap, &q));
+    else if (!direct)
+        LV_TRY(tc_reserve(ws, fdt == LUDVIG_F32 ? 2 : 1, nv * TX * TY, s->tc_chunk_cap, sets));
     const int64_t npx = (int64_t)nv * width * height;
     for (int p = 0; p < sets; ++p) {
         static const char* const kFb[2] = {"fp8.bf16.0", "fp8.bf16.1"};
@@ -1556,7 +1586,7 @@ ludvig_status size_for_async(ludvig_scene* s, const std::vector<GroupViews>& gro
                              const FeatSrc& src, bool tc, bool always, cudaStream_t st, size_t* first) {
     *first = 0;
     if (groups.empty()) return LUDVIG_OK;
-    if (always || s->pair_cap == 0 || (!src_direct(src) && s->tc_chunk_cap == 0)) {
+    if (always || s->pair_cap == 0 || (tc && !src_direct(src) && s->tc_chunk_cap == 0)) {
         const int64_t pc0 = s->pair_cap, cc0 = s->tc_chunk_cap;
         LV_TRY(run_checked(s, groups[0], width, height, src, st));
         if (s->pair_cap > pc0) s->pair_cap = round_up(s->pair_cap + s->pair_cap / 4, kRadixTile);
@@ -2144,6 +2174,16 @@ extern "C" ludvig_status ludvig_debug_transmittance(ludvig_scene_t scene, const 
     if (scene->n == 0) return LUDVIG_OK;
     LV_TRY(ensure_status(scene));
     LV_TRY(resolve_pending(scene));
+    float* num;
+    float* den;
+    LV_TRY(scene->ws.get("dbg.num", (size_t)scene->n, &num));
+    LV_TRY(scene->ws.get("dbg.den", (size_t)scene->n, &den));
+    float* fz;
+    LV_TRY(scene->ws.get("dbg.feat", (size_t)npx, &fz));
+    LV_CUDA(cudaMemsetAsync(fz, 0, sizeof(float) * npx, st));
+    ChunkDebug dbg;
+    dbg.t_final = t_final;
+    dbg.n_contrib = n_contrib;
     FrontEnd fe;
     LV_TRY(front_end(scene, scene_group(scene, cam, 0, 1, nullptr, nullptr), width, height, true, nullptr, nullptr,
                      st, &fe));
@@ -2151,13 +2191,5 @@ extern "C" ludvig_status ludvig_debug_transmittance(ludvig_scene_t scene, const 
         set_error("too many pairs");
         return LUDVIG_ERR_UNSUPPORTED;
     }
-    const int TX = (width + kTile - 1) / kTile, ntiles = TX * ((height + kTile - 1) / kTile);
-    PairRec* pairs;
-    LV_TRY(scene->ws.get("up.pairs", (size_t)fe.cap, &pairs));
-    k_pair_records<<<kPairGrid, 256, 0, st>>>(fe.spk, fe.L.rank, fe.np, (uint64_t)fe.cap, ntiles, TX, fe.L.npad,
-                                              fe.L.srec, pairs);
-    LV_LAUNCH();
-    k_transmittance<<<(unsigned)ntiles, 256, 0, st>>>(pairs, fe.L.ranges, TX, width, height, t_final, n_contrib);
-    LV_LAUNCH();
-    return LUDVIG_OK;
+    return composite_cc(scene, fe, 1, width, height, fz, LUDVIG_F32, 1, num, den, &dbg, st);
 }

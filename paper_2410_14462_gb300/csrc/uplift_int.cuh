@@ -104,7 +104,7 @@ struct TileWeights {
     int64_t cap = 0;          // chunks the buffers hold
     int count = -1;           // chunks used, when read back by a checked run (else -1)
     int* counter = nullptr;   // device: chunks used
-    uint8_t *wg1 = nullptr, *wg2 = nullptr;   // bfloat16 rows of one or two terms, or (NT = 3) float32 rows in wg1
+    uint8_t *wg1 = nullptr, *wg2 = nullptr;
     uint32_t* cgid = nullptr;
     int *crows = nullptr, *cnext = nullptr, *ifirst = nullptr;
     float* cden = nullptr;

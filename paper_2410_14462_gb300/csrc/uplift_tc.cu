@@ -88,7 +88,7 @@ struct WeightsArgs {
     int64_t npad;
     const uint2* ranges;
     int ntiles, TX, width, height;
-    uint8_t* wg1;           // [cap][128][256] bfloat16: W (NT = 1) or W1; float32: W (NT = 3)
+    uint8_t* wg1;           // [cap][128][256] bfloat16: W (NT = 1) or W1
     uint8_t* wg2;           // W2 (NT = 2)
     uint32_t* chunk_gid;    // [cap][128]
     int* chunk_rows;        // [cap]
@@ -96,7 +96,7 @@ struct WeightsArgs {
     int* item_first;        // [nitems]: the tile's first chunk, or -1 (set to -1 before the launch)
     int* chunk_counter;
     int cap;
-    float* chunk_den;       // [cap][128][1, or 2 for NT = 2]: each row's den, the sum of its weight terms, in term 0's
+    float* chunk_den;       // [cap][128][NT]: each row's den, the sum of its weight terms, in term 0's
                             // slot (term 1's: 0); rewritten on a re-run
     // direct accumulation (k_weights<NT, true>, few channels): each new row's
     // sum_p w F[p, c] and its den go straight into the view's num and den
@@ -126,7 +126,7 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
 // The weights of one (view, tile), a warp per tile (NB = 4) or per 8x8 quadrant
 // of it (NB = 1); a lane holds two neighbouring pixels of each quadrant.
 //   DD = 0: weight rows; DD = 1 .. 4: direct accumulation of DD channels.
-//   NT = 1, 2: weights as one or two bfloat16 terms; 3: float32 rows.
+//   NT = 1, 2: weights as one or two bfloat16 terms.
 //   COUNT: den is the number of a row's non-zero weights instead of their sum.
 //
 // Bound: instruction issue (0.74 of it, FMA pipe and ALU half busy each), with
@@ -152,8 +152,7 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
 template <int NT, int DD, int NB, bool COUNT>
 __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_constant__ WeightsArgs a) {
     constexpr bool kDirect = DD > 0;
-    constexpr int kPx = NT == 3 ? 4 : 2;           // bytes per pixel of a row
-    constexpr int kDen = NT == 2 ? 2 : 1;          // den slots per row
+    constexpr int kPx = 2;                        // bytes per pixel of a row
     constexpr int kVals = kDirect ? DD + 1 : 1;   // sums per row
     constexpr int kRowBuf = 32 / kVals;           // rows whose lane sums are kept
     constexpr int kGroup = NB == 1 ? 2 : 1;       // entries taken together (a row is one entry's: NB = 4 takes one)
@@ -357,9 +356,7 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                         const float wx = tn.x >= kTransMin ? ww.x : 0.f, wy = tn.y >= kTransMin ? ww.y : 0.f;
                         nz |= __float_as_uint(wx) | __float_as_uint(wy);
                         F2 wv = f2(wx, wy);
-                        if (NT == 3) {
-                            *reinterpret_cast<float2*>(d1 + kQuadByte(b)) = make_float2(wx, wy);
-                        } else if (!kDirect || NT == 1) {
+                        if (!kDirect || NT == 1) {
                             const __nv_bfloat162 h = __floats2bfloat162_rn(wx, wy);
                             const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
                             const F2 hf = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u));
@@ -387,8 +384,6 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                         auto quad_or_zero = [&](int b) {
                             if (B[b] & bit) {
                                 finish(b, alpha(g, b));
-                            } else if (NT == 3) {
-                                *reinterpret_cast<float2*>(d1 + kQuadByte(b)) = make_float2(0.f, 0.f);
                             } else if (!kDirect) {
                                 *reinterpret_cast<uint32_t*>(d1 + kQuadByte(b)) = 0u;
                                 if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + kQuadByte(b)) = 0u;
@@ -449,8 +444,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
             if (((rowbits >> lane) & 1u) && myrow >= 0) {
                 const float s = lane_sum(__popc(rowbits & lt_mask));
                 // the row's den in term 0's slot (the aggregation adds the slots)
-                a.chunk_den[(size_t)myrow * kDen] = s;
-                if (NT == 2) a.chunk_den[(size_t)myrow * kDen + 1] = 0.f;
+                a.chunk_den[(size_t)myrow * NT] = s;
+                if (NT == 2) a.chunk_den[(size_t)myrow * NT + 1] = 0.f;
                 a.chunk_gid[myrow] = gid;
             }
             nbuf = 0;
@@ -1830,17 +1825,13 @@ const char* const kWsCounter[2] = {"tc.counter.0", "tc.counter.1"};
 const char* const kWsPlanOff[2] = {"tc.plan_off.0", "tc.plan_off.1"};
 const char* const kWsPlan[2] = {"tc.plan.0", "tc.plan.1"};
 
-// Chunks a group's weight rows start with: three per tile (380 rows).  Float32
-// rows serve small images more often, whose tiles hold more Gaussians: four.
-int64_t start_chunks(int NT, int nitems) { return (NT == 3 ? 4 : 3) * (int64_t)nitems; }
-
 ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets) {
-    cap = std::max<int64_t>(cap, start_chunks(NT, nitems));
+    cap = std::max<int64_t>(cap, 3 * (int64_t)nitems);
     for (int p = 0; p < sets; ++p) {
         void* q;
         LV_TRY(ws.get(kWsCounter[p], sizeof(int), &q));
         LV_TRY(ws.get(kWsFirst[p], sizeof(int) * (size_t)nitems, &q));
-        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes * (NT == 3 ? 2 : 1), &q));
+        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes, &q));
         if (NT == 2) LV_TRY(ws.get(kWsW2[p], (size_t)cap * kChunkBytes, &q));
         LV_TRY(ws.get(kWsGid[p], sizeof(uint32_t) * (size_t)cap * kCRows, &q));
         LV_TRY(ws.get(kWsRows[p], sizeof(int) * (size_t)cap, &q));
@@ -1856,13 +1847,10 @@ namespace {
 template <int NT>
 void launch_weight_rows(const WeightsArgs& w, int nitems, cudaStream_t st) {
     const bool count = option_count_normalise();
-    if constexpr (NT != 3) {
-        if (nitems < kBlockItems) {
-            count ? k_weights_block<NT, true><<<nitems, 256, 0, st>>>(w) : k_weights_block<NT, false><<<nitems, 256, 0, st>>>(w);
-            return;
-        }
-    }
-    count ? k_weights<NT, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<NT, 0, 4, false><<<nitems, 32, 0, st>>>(w);
+    if (nitems < kBlockItems)
+        count ? k_weights_block<NT, true><<<nitems, 256, 0, st>>>(w) : k_weights_block<NT, false><<<nitems, 256, 0, st>>>(w);
+    else
+        count ? k_weights<NT, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<NT, 0, 4, false><<<nitems, 32, 0, st>>>(w);
 }
 }  // namespace
 
@@ -1880,13 +1868,13 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         LV_TRY(ws.pinned("tc.host", 16, &hp));
         host = static_cast<int*>(hp);
     }
-    int64_t cap = std::max<int64_t>(*chunk_cap, start_chunks(NT, nitems));
+    int64_t cap = std::max<int64_t>(*chunk_cap, 3 * (int64_t)nitems);
     for (int attempt = 0; attempt < 2; ++attempt) {
         if (cap > 0x7fffffff / kCRows) {
             set_error("tile weights need %lld chunks of 128 rows", (long long)cap);
             return LUDVIG_ERR_UNSUPPORTED;
         }
-        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes * (NT == 3 ? 2 : 1), &t.wg1));
+        LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes, &t.wg1));
         if (NT == 2) LV_TRY(ws.get(kWsW2[p], (size_t)cap * kChunkBytes, &t.wg2));
         LV_TRY(ws.get(kWsGid[p], (size_t)cap * kCRows, &t.cgid));
         LV_TRY(ws.get(kWsRows[p], (size_t)cap, &t.crows));
@@ -1914,9 +1902,7 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         w.chunk_den = t.cden;
         w.one = make_float2(1.f, 1.f);
         const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
-        if (NT == 3)
-            launch_weight_rows<3>(w, nitems, st);
-        else if (NT == 2)
+        if (NT == 2)
             launch_weight_rows<2>(w, nitems, st);
         else
             launch_weight_rows<1>(w, nitems, st);

@@ -92,3 +92,17 @@ def test_centres_not_finite_leave_the_graph_alone():
         ref = r.diffuse(torch.from_numpy(xs[good]).cuda(), 5).cpu().numpy()
         assert np.all(got[bad] == 0)
         assert rel_l2(got[good], ref) <= 1e-5
+
+
+@pytest.mark.parametrize("d,dtype", [(33, torch.float32), (100, torch.bfloat16), (520, torch.float32)])
+def test_cuda_core_widths_keep_no_weight_rows(d, dtype):
+    """The scratch of such a call is its (tile, Gaussian) lists and a 32-byte record per
+    pair, about what a call of three channels holds, whose walk writes no rows either."""
+    wl = inputs.small_field_workload(n=50_000, views=3, d=d, width=320, height=240)
+    size = []
+    for c in (3, d):
+        sc = ludvig.Scene.from_inputs(wl.scene)
+        F = torch.rand((3, 240, 320, c), device="cuda").to(dtype)
+        ludvig.uplift(sc, wl.cams.params, 320, 240, F)
+        size.append(sc.workspace_bytes())
+    assert size[1] <= 3 * size[0], size
