@@ -109,16 +109,6 @@ __global__ void k_cell_keys(const float* __restrict__ x, int64_t n, int64_t npad
     vals[i] = (uint32_t)i;
 }
 
-// start[c] = the first sorted position whose cell is >= c (so cell c holds
-// [start[c], start[c + 1]), and a run of cells along x one range).
-__global__ void k_cell_starts(const uint32_t* __restrict__ keys, int64_t n, int64_t ncell,
-                              uint32_t* __restrict__ start) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j > n) return;
-    const int64_t lo = j == 0 ? 0 : (int64_t)keys[j - 1] + 1, hi = j == n ? ncell : (int64_t)keys[j];
-    for (int64_t c = lo; c <= hi; ++c) start[c] = (uint32_t)j;
-}
-
 // Points sorted by cell are stored as float4 (x, y, z, index) in cell order.
 __global__ void k_gather_sorted(const float* __restrict__ x, const uint32_t* __restrict__ order,
                                 int64_t n, float4* __restrict__ pts) {
@@ -993,17 +983,22 @@ ludvig_status knn_impl(ludvig_scene* s, int k, int32_t* nbr, cudaStream_t st, co
         // mean over the points, 3 for uniform points).  Clustered scenes leave
         // most cells empty: at 6 points the search of 1M clustered centres takes
         // 2.3 ms (3: 3.2, 12: 2.3, cells as they are: 2.9)
-        if (n >= kKnnDensityMin) {
-            uint32_t* cc;
-            unsigned long long* sq;
-            const int64_t nc = cells_of(cell);
-            LV_TRY(ws.get("knn.count", (size_t)nc, &cc));
-            LV_TRY(ws.get("knn.sq", 1, &sq));
-            LV_CUDA(cudaMemsetAsync(cc, 0, sizeof(uint32_t) * (size_t)nc, st));
-            LV_CUDA(cudaMemsetAsync(sq, 0, sizeof(unsigned long long), st));
-            k_cell_count<<<grid_for(n, 256), 256, 0, st>>>(s->means, n, gr, cc);
+        int64_t ncell = 0;
+        uint32_t* cells = nullptr;
+        const auto count_cells = [&]() -> ludvig_status {   // and a zero behind the last
+            ncell = (int64_t)gr.g[0] * gr.g[1] * gr.g[2];
+            LV_TRY(ws.get("knn.cells", (size_t)ncell + 1, &cells));
+            LV_CUDA(cudaMemsetAsync(cells, 0, sizeof(uint32_t) * ((size_t)ncell + 1), st));
+            k_cell_count<<<grid_for(n, 256), 256, 0, st>>>(s->means, n, gr, cells);
             LV_LAUNCH();
-            k_cell_square<<<(unsigned)std::min<int64_t>(608, ceil_div(nc, 256)), 256, 0, st>>>(cc, nc, sq);
+            return LUDVIG_OK;
+        };
+        LV_TRY(count_cells());
+        if (n >= kKnnDensityMin) {
+            unsigned long long* sq;
+            LV_TRY(ws.get("knn.sq", 1, &sq));
+            LV_CUDA(cudaMemsetAsync(sq, 0, sizeof(unsigned long long), st));
+            k_cell_square<<<(unsigned)std::min<int64_t>(608, ceil_div(ncell, 256)), 256, 0, st>>>(cells, ncell, sq);
             LV_LAUNCH();
             LV_CUDA(cudaMemcpyAsync(static_cast<char*>(h) + 56, sq, 8, cudaMemcpyDeviceToHost, st));
             LV_CUDA(cudaStreamSynchronize(st));
@@ -1018,10 +1013,15 @@ ludvig_status knn_impl(ludvig_scene* s, int k, int32_t* nbr, cudaStream_t st, co
                 if (c < cell) {
                     cell = c;
                     set_grid(cell);
+                    LV_TRY(count_cells());
                 }
             }
         }
-        const int64_t ncell = (int64_t)gr.g[0] * gr.g[1] * gr.g[2];
+        // cells[c] = the first sorted position of cell c (a run of cells along x is one
+        // range): the counts' prefix, whose time does not depend on how the empty cells
+        // lie (a thread that wrote the gap before its point took 45 ms for two
+        // tight clusters far apart, 100k points)
+        LV_TRY(scan_exclusive_u32(cells, cells, ncell + 1, nullptr, ws, st));
         const int64_t npad = round_up(n, kRadixTile);
         uint32_t *keys, *vals, *keys2, *vals2;
         LV_TRY(ws.get("knn.keys", (size_t)npad, &keys));
@@ -1034,10 +1034,6 @@ ludvig_status knn_impl(ludvig_scene* s, int k, int32_t* nbr, cudaStream_t st, co
         while (((int64_t)1 << nbits) <= ncell) ++nbits;
         uint32_t *sk = keys, *sv = vals;
         LV_TRY(radix_sort_pairs(&sk, &sv, keys2, vals2, 1, npad, nbits, ws, st));
-        uint32_t* cells;
-        LV_TRY(ws.get("knn.cells", (size_t)ncell + 1, &cells));
-        k_cell_starts<<<grid_for(n + 1, 256), 256, 0, st>>>(sk, n, ncell, cells);
-        LV_LAUNCH();
         float4* pts;
         LV_TRY(ws.get("knn.pts", (size_t)n, &pts));
         k_gather_sorted<<<grid_for(n, 256), 256, 0, st>>>(s->means, sv, n, pts);
