@@ -5,7 +5,9 @@
 // kNN: points are bucketed in a uniform grid (cells sorted by the radix sort);
 // one thread per query scans the 27 cells around its own, then ring by ring
 // (Chebyshev distance r), and stops once the k-th best squared distance is below
-// the squared gap r*cell to the unvisited rings.  Squared distances are float32
+// the squared gap r*cell to the unvisited rings.  A query whose neighbours lie
+// more than a few rings away goes on by itself in a warp, by blocks of 8x8x8
+// cells (k_knn_far).  Squared distances are float32
 // (dx*dx + dy*dy) + dz*dz with d = x_j - x_i and ties go to the lower index,
 // so the result is exact and independent of the scan order.
 //
@@ -92,6 +94,13 @@ __global__ void k_cell_square(const uint32_t* __restrict__ cnt, int64_t nc, unsi
 
 constexpr double kKnnCellPoints = 6.0;       // points a point should find in its cell
 constexpr int64_t kKnnDensityMin = 1 << 14;  // below, the pass over the counts costs more than it saves
+// Rings a thread searches by itself: most points are done after two or three of
+// them, and a wider search is a chain of reads that its warp waits for.  Limits of
+// 4, 6, 8 and 12 (ms, k = 16): 100k clustered centres 0.84, 0.65, 0.66, 0.66, 200 of them
+// moved far out 1.24, 1.25, 1.44, 2.75; 1M centres, a tenth of them in a wide
+// shell, 9.4, 8.5, 7.9, 7.8.
+constexpr int kKnnNear = 8;
+constexpr int kKnnBlock = 8;                 // cells along each axis of a block of cells
 
 __global__ void k_cell_keys(const float* __restrict__ x, int64_t n, int64_t npad, Grid gr,
                             uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
@@ -136,11 +145,16 @@ __device__ __forceinline__ void knn_insert(uint64_t (&best)[K], uint64_t key) {
 template <int K>
 __global__ void __launch_bounds__(128) k_knn(const float4* __restrict__ pts, int64_t n, Grid gr,
                                              const uint32_t* __restrict__ start, int k,
-                                             int32_t* __restrict__ out) {
+                                             int32_t* __restrict__ out, uint32_t* __restrict__ far,
+                                             uint32_t* __restrict__ nfar) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const float4 q = pts[j];
     const uint32_t qi = __float_as_uint(q.w);
+    if (!(isfinite(q.x) && isfinite(q.y) && isfinite(q.z))) {   // at no finite distance from any point
+        for (int t = 0; t < k; ++t) out[(int64_t)qi * k + t] = -1;
+        return;
+    }
     // the best so far, ascending: squared distance (its bits order like the
     // value), then index; K - k entries that nothing precedes fill the list up,
     // so that the k-th best is always the last
@@ -152,7 +166,8 @@ __global__ void __launch_bounds__(128) k_knn(const float4* __restrict__ pts, int
     const int cy = cell_coord(q.y, gr.lo[1], gr.inv_cell, gr.g[1]);
     const int cz = cell_coord(q.z, gr.lo[2], gr.inv_cell, gr.g[2]);
     const int rmax = max(gr.g[0], max(gr.g[1], gr.g[2]));
-    for (int r = 1; r <= max(1, rmax); ++r) {
+    bool found = rmax <= kKnnNear;   // (the last ring ends that search)
+    for (int r = 1; r <= min(max(1, rmax), kKnnNear); ++r) {
         for (int dz = -r; dz <= r; ++dz) {
             const int z = cz + dz;
             if (z < 0 || z >= gr.g[2]) continue;
@@ -184,11 +199,164 @@ __global__ void __launch_bounds__(128) k_knn(const float4* __restrict__ pts, int
         const uint64_t kth = best[K - 1];
         const float gap = (float)r * gr.cell;
         // 0.1% margin: rounding can put a point next to a cell border in the neighbour cell
-        if (kth != kNone && __uint_as_float((uint32_t)(kth >> 32)) < gap * gap * 0.999f) break;
+        if (kth != kNone && __uint_as_float((uint32_t)(kth >> 32)) < gap * gap * 0.999f) {
+            found = true;
+            break;
+        }
+    }
+    if (!found) {   // (k_knn_far starts afresh)
+        far[atomicAdd(nfar, 1u)] = (uint32_t)j;
+        return;
     }
 #pragma unroll
     for (int t = 0; t < K; ++t)
         if (t >= K - k) out[(int64_t)qi * k + (t - (K - k))] = best[t] == kNone ? -1 : (int32_t)(uint32_t)best[t];
+}
+
+// ---- queries far from their neighbours
+// The points in every block of 8x8x8 cells (bg blocks along each axis).
+__global__ void k_block_count(const uint32_t* __restrict__ start, Grid gr, int3 bg, int64_t nblocks,
+                              const uint32_t* __restrict__ nfar, uint32_t* __restrict__ cnt) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nblocks || *nfar == 0u) return;
+    const int bx = (int)(t % bg.x), by = (int)(t / bg.x % bg.y), bz = (int)(t / bg.x / bg.y);
+    const int x0 = bx * kKnnBlock, x1 = min(x0 + kKnnBlock, gr.g[0]);
+    uint32_t c = 0;
+    for (int z = bz * kKnnBlock; z < min((bz + 1) * kKnnBlock, gr.g[2]); ++z)
+        for (int y = by * kKnnBlock; y < min((by + 1) * kKnnBlock, gr.g[1]); ++y) {
+            const uint32_t* row = start + ((int64_t)z * gr.g[1] + y) * gr.g[0];
+            c += row[x1] - row[x0];
+        }
+    cnt[t] = c;
+}
+
+// One warp per query of the list `far`, its k best so far in ascending order
+// over the lanes (entry t is list[t / 32] of lane t % 32).  The blocks of cells
+// are visited in Chebyshev rings around the query's own (ring R's six faces, 32
+// blocks at a time); empty ones, and those further away than the k-th best, cost
+// their share of one read, the others are scanned by the whole warp.  Bound by
+// the latency of those reads.  The whole search, k = 16: 100k clustered centres of
+// which 8 lie far out 1.7 ms, 1M 23.6 (2490 and 3020 with one thread walking all rings
+// of cells); 200 of them anywhere in a wide box 1.4 and 8.3 (431 and 1170).
+template <int P>
+__global__ void __launch_bounds__(128) k_knn_far(const float4* __restrict__ pts, Grid gr,
+                                                 const uint32_t* __restrict__ start, int3 bg,
+                                                 const uint32_t* __restrict__ bcnt, int k,
+                                                 const uint32_t* __restrict__ far, const uint32_t* __restrict__ nfar,
+                                                 int32_t* __restrict__ out) {
+    constexpr uint32_t kAll = 0xffffffffu;
+    constexpr uint64_t kNone = ~0ull;
+    const int lane = threadIdx.x & 31;
+    const uint32_t nq = *nfar, nwarps = gridDim.x * (blockDim.x >> 5);
+    // cells by which a coordinate divided by the cell's size may be off, twice (the
+    // query's and the point's)
+    const float slack = 0.01f + 1e-6f * (float)max(gr.g[0], max(gr.g[1], gr.g[2]));
+    for (uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nq; w += nwarps) {
+        const float4 q = pts[far[w]];
+        const uint32_t qi = __float_as_uint(q.w);
+        const float u[3] = {(q.x - gr.lo[0]) * gr.inv_cell, (q.y - gr.lo[1]) * gr.inv_cell,
+                            (q.z - gr.lo[2]) * gr.inv_cell};
+        const int b[3] = {cell_coord(q.x, gr.lo[0], gr.inv_cell, gr.g[0]) / kKnnBlock,
+                          cell_coord(q.y, gr.lo[1], gr.inv_cell, gr.g[1]) / kKnnBlock,
+                          cell_coord(q.z, gr.lo[2], gr.inv_cell, gr.g[2]) / kKnnBlock};
+        uint64_t list[P], kth = kNone;
+#pragma unroll
+        for (int e = 0; e < P; ++e) list[e] = kNone;
+        auto kth_dist = [&]() { return __uint_as_float((uint32_t)(kth >> 32)); };
+        auto insert = [&](uint64_t key) {
+            uint64_t below = 0ull;   // the entry before lane 0's
+#pragma unroll
+            for (int e = 0; e < P; ++e) {
+                uint64_t left = __shfl_up_sync(kAll, list[e], 1);
+                const uint64_t last = __shfl_sync(kAll, list[e], 31);
+                if (lane == 0) left = below;
+                below = last;
+                list[e] = key < list[e] ? (key > left ? key : left) : list[e];
+            }
+#pragma unroll
+            for (int e = 0; e < P; ++e)
+                if ((k - 1) / 32 == e) kth = __shfl_sync(kAll, list[e], (k - 1) & 31);
+        };
+        // could the block at (x, y, z) hold one of the k?
+        auto reaches = [&](int x, int y, int z) {
+            const int c[3] = {x, y, z};
+            float d2 = 0.f;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float l = (float)(c[a] * kKnnBlock);
+                const float t = fmaxf(fmaxf(l - u[a], u[a] - (l + (float)kKnnBlock)) - slack, 0.f) * gr.cell;
+                d2 += t * t;
+            }
+            return kth == kNone || d2 * 0.999f <= kth_dist();
+        };
+        auto scan_block = [&](int x, int y, int z) {
+            const int x0 = x * kKnnBlock, x1 = min(x0 + kKnnBlock, gr.g[0]);
+#pragma unroll 1
+            for (int h = 0; h < kKnnBlock * kKnnBlock; h += 32) {
+                const int ry = y * kKnnBlock + ((h + lane) & (kKnnBlock - 1)), rz = z * kKnnBlock + (h + lane) / kKnnBlock;
+                uint32_t p0 = 0u, p1 = 0u;
+                if (ry < gr.g[1] && rz < gr.g[2]) {
+                    const uint32_t* row = start + ((int64_t)rz * gr.g[1] + ry) * gr.g[0];
+                    p0 = row[x0];
+                    p1 = row[x1];
+                }
+                for (uint32_t m = __ballot_sync(kAll, p1 > p0); m; m &= m - 1u) {
+                    const int src = __ffs(m) - 1;
+                    const uint32_t s0 = __shfl_sync(kAll, p0, src), s1 = __shfl_sync(kAll, p1, src);
+                    for (uint32_t s = s0; s < s1; s += 32) {
+                        uint64_t key = kNone;
+                        if (s + lane < s1) {
+                            const float4 c = pts[s + lane];
+                            const uint32_t ci = __float_as_uint(c.w);
+                            const float ex = __fsub_rn(c.x, q.x), ey = __fsub_rn(c.y, q.y), ez = __fsub_rn(c.z, q.z);
+                            const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
+                            if (ci != qi && d2 <= FLT_MAX) key = ((uint64_t)__float_as_uint(d2) << 32) | ci;
+                        }
+                        for (uint32_t c = __ballot_sync(kAll, key < kth); c; c &= c - 1u) {
+                            const uint64_t kk = __shfl_sync(kAll, key, __ffs(c) - 1);
+                            if (kk < kth) insert(kk);
+                        }
+                    }
+                }
+            }
+        };
+        const int rmax = max(max(max(b[0], bg.x - 1 - b[0]), max(b[1], bg.y - 1 - b[1])), max(b[2], bg.z - 1 - b[2]));
+        for (int r = 0; r <= rmax; ++r) {
+            const int xl = max(b[0] - r, 0), xh = min(b[0] + r, bg.x - 1);
+            const int yl = max(b[1] - r, 0), yh = min(b[1] + r, bg.y - 1);
+            const int yi = max(b[1] - r + 1, 0), yj = min(b[1] + r - 1, bg.y - 1);
+            const int zi = max(b[2] - r + 1, 0), zj = min(b[2] + r - 1, bg.z - 1);
+#pragma unroll 1
+            for (int f = 0; f < (r == 0 ? 1 : 6); ++f) {
+                // the faces across z whole, those across y without the first, those across x without both
+                const int axis = 2 - (f >> 1), at = b[axis] + ((f & 1) ? r : -r);
+                if (at < 0 || at >= (axis == 0 ? bg.x : axis == 1 ? bg.y : bg.z)) continue;
+                const int x0 = axis == 0 ? at : xl, nx = axis == 0 ? 1 : xh - xl + 1;
+                const int y0 = axis == 1 ? at : axis == 0 ? yi : yl, ny = axis == 1 ? 1 : axis == 0 ? yj - yi + 1 : yh - yl + 1;
+                const int z0 = axis == 2 ? at : zi, nz = axis == 2 ? 1 : zj - zi + 1;
+                if (nx <= 0 || ny <= 0 || nz <= 0) continue;
+                const int total = nx * ny * nz;   // (a grid has at most 2^24 cells)
+                for (int t0 = 0; t0 < total; t0 += 32) {
+                    const int t = t0 + lane, line = t / nx;
+                    const int x = x0 + t - line * nx, y = y0 + line % ny, z = z0 + line / ny;
+                    const bool in = t < total && bcnt[((int64_t)z * bg.y + y) * bg.x + x] > 0u && reaches(x, y, z);
+                    for (uint32_t m = __ballot_sync(kAll, in); m; m &= m - 1u) {
+                        const int src = __ffs(m) - 1;
+                        const int sx = __shfl_sync(kAll, x, src), sy = __shfl_sync(kAll, y, src),
+                                  sz = __shfl_sync(kAll, z, src);
+                        if (reaches(sx, sy, sz)) scan_block(sx, sy, sz);   // (the k-th best may have come nearer)
+                    }
+                }
+            }
+            // every point outside the visited blocks is at least r blocks away
+            const float gap = fmaxf((float)(r * kKnnBlock) - slack, 0.f) * gr.cell;
+            if (kth != kNone && kth_dist() < gap * gap * 0.999f) break;
+        }
+#pragma unroll
+        for (int e = 0; e < P; ++e)
+            if (32 * e + lane < k)
+                out[(int64_t)qi * k + 32 * e + lane] = list[e] == kNone ? -1 : (int32_t)(uint32_t)list[e];
+    }
 }
 
 // ------------------------------------------------------------ graph build
@@ -985,10 +1153,10 @@ ludvig_status knn_impl(ludvig_scene* s, int k, int32_t* nbr, cudaStream_t st, co
         // 2.3 ms (3: 3.2, 12: 2.3, cells as they are: 2.9)
         int64_t ncell = 0;
         uint32_t* cells = nullptr;
-        const auto count_cells = [&]() -> ludvig_status {   // and a zero behind the last
+        const auto count_cells = [&]() -> ludvig_status {   // and two zeros behind the last
             ncell = (int64_t)gr.g[0] * gr.g[1] * gr.g[2];
-            LV_TRY(ws.get("knn.cells", (size_t)ncell + 1, &cells));
-            LV_CUDA(cudaMemsetAsync(cells, 0, sizeof(uint32_t) * ((size_t)ncell + 1), st));
+            LV_TRY(ws.get("knn.cells", (size_t)ncell + 2, &cells));
+            LV_CUDA(cudaMemsetAsync(cells, 0, sizeof(uint32_t) * ((size_t)ncell + 2), st));
             k_cell_count<<<grid_for(n, 256), 256, 0, st>>>(s->means, n, gr, cells);
             LV_LAUNCH();
             return LUDVIG_OK;
@@ -1039,11 +1207,25 @@ ludvig_status knn_impl(ludvig_scene* s, int k, int32_t* nbr, cudaStream_t st, co
         k_gather_sorted<<<grid_for(n, 256), 256, 0, st>>>(s->means, sv, n, pts);
         LV_LAUNCH();
         const unsigned g = grid_for(n, 128);
-        if (k <= 8) k_knn<8><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr);
-        else if (k <= 16) k_knn<16><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr);
-        else if (k <= 32) k_knn<32><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr);
-        else k_knn<64><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr);
+        uint32_t *far = sk, *nfar = cells + ncell + 1;   // (the sorted keys are used up; a zero behind the starts)
+        if (k <= 8) k_knn<8><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr, far, nfar);
+        else if (k <= 16) k_knn<16><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr, far, nfar);
+        else if (k <= 32) k_knn<32><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr, far, nfar);
+        else k_knn<64><<<g, 128, 0, st>>>(pts, n, gr, cells, k, nbr, far, nfar);
         LV_LAUNCH();
+        if (std::max(gr.g[0], std::max(gr.g[1], gr.g[2])) > kKnnNear) {   // (else every search has ended)
+            const int3 bg = make_int3((gr.g[0] + kKnnBlock - 1) / kKnnBlock, (gr.g[1] + kKnnBlock - 1) / kKnnBlock,
+                                      (gr.g[2] + kKnnBlock - 1) / kKnnBlock);
+            const int64_t nblocks = (int64_t)bg.x * bg.y * bg.z;
+            uint32_t* bcnt;
+            LV_TRY(ws.get("knn.blocks", (size_t)nblocks, &bcnt));
+            k_block_count<<<grid_for(nblocks, 256), 256, 0, st>>>(cells, gr, bg, nblocks, nfar, bcnt);
+            LV_LAUNCH();
+            const unsigned gf = (unsigned)std::min<int64_t>(ceil_div(n, 4), 152 * 16);
+            if (k <= 32) k_knn_far<1><<<gf, 128, 0, st>>>(pts, gr, cells, bg, bcnt, k, far, nfar, nbr);
+            else k_knn_far<2><<<gf, 128, 0, st>>>(pts, gr, cells, bg, bcnt, k, far, nfar, nbr);
+            LV_LAUNCH();
+        }
         if (order) {
             int shift = 0;
             while ((std::max(gr.g[0], std::max(gr.g[1], gr.g[2])) >> shift) > 1024) ++shift;

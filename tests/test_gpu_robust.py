@@ -116,7 +116,7 @@ def _two_clusters(n):
     return m.astype(np.float32)
 
 
-def _knn_seconds(sc, k):
+def _knn_ms(sc, k):
     ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
     best = float("inf")
     for _ in range(4):   # the first call allocates
@@ -138,4 +138,37 @@ def test_knn_of_far_clusters(n, k):
 def test_knn_time_does_not_depend_on_where_cells_are_empty():
     """A hundred thousand points take under 10 ms (4.7 on a GB300) where the
     empty cells between two clusters, written by one thread, alone took 48."""
-    assert _knn_seconds(ludvig.Scene.from_inputs(_scene_at(_two_clusters(100_000))), 16) <= 10.0
+    assert _knn_ms(ludvig.Scene.from_inputs(_scene_at(_two_clusters(100_000))), 16) <= 10.0
+
+
+def _far_points(kind, n):
+    """Clustered centres, some of them moved far out: the corners of a box many times
+    as wide, a few anywhere in it, or a wide shell of a tenth of them."""
+    rng = np.random.default_rng(7)
+    m = inputs.scene_clusters(n, seed=1).means.astype(np.float64)
+    if kind == "corners":
+        m[:8] = 20.0 * np.array([[x, y, z] for x in (-1, 1) for y in (-1, 1) for z in (-1, 1)]) + rng.normal(size=(8, 3))
+    elif kind == "sparse":
+        m[:200] = rng.uniform(-5, 5, size=(200, 3)) * np.abs(m).max()
+    elif kind == "shell":
+        d = rng.normal(size=(n // 10, 3))
+        m[:n // 10] = d / np.linalg.norm(d, axis=1, keepdims=True) * rng.uniform(8, 12, size=(n // 10, 1))
+    else:   # all but on a line, so that one axis has nearly all cells
+        m *= np.array([50.0, 1e-3, 1e-3])
+        m[:3, 0] += 900.0
+    return m.astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["corners", "sparse", "shell", "line"])
+@pytest.mark.parametrize("n,k", [(3000, 64), (20_000, 16), (40_000, 33), (30, 32), (5000, 1)])
+def test_knn_of_far_points(kind, n, k):
+    m = _far_points(kind, n) if n >= 3000 else _far_points(kind, 3000)[:n]
+    got = ludvig.knn(ludvig.Scene.from_inputs(_scene_at(m)), k).cpu().numpy()
+    assert np.array_equal(got, oracle.knn(m, k)[0])
+
+
+@pytest.mark.parametrize("kind", ["corners", "sparse"])
+def test_knn_time_with_far_points(kind):
+    """A few points far from all others do not hold up the search of a hundred
+    thousand (2490 and 431 ms where one thread walked all rings of cells)."""
+    assert _knn_ms(ludvig.Scene.from_inputs(_scene_at(_far_points(kind, 100_000))), 16) <= 40.0
