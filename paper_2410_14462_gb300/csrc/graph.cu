@@ -840,41 +840,13 @@ __device__ __forceinline__ Ent4 load_ent4(const int2* p) {
     return r;
 }
 
-// A sum of squares over the whole float32 range, to about 2^-46, in float32
-// arithmetic: the values are scaled by a power of two that keeps the largest
-// one so far at or below 1, and the products and the additions keep their
-// rounding errors (Dekker's and Knuth's exact forms).  Summing in float64 would
-// cost a step more than its gathers do: those units run at a 64th of the rate.
-struct SumSq {
-    float s = 0.f, c = 0.f, scale = 0x1p126f;
-    __device__ __forceinline__ void add(float a) {
-        if (fabsf(a) * scale > 1.f) {   // a new largest value (rare)
-            const int e = (int)((__float_as_uint(a) >> 23) & 255u);
-            const float ns = __uint_as_float((uint32_t)max(1, 253 - e) << 23);
-            const float f = ns / scale;   // a power of two, or 0
-            s *= f * f;
-            c *= f * f;
-            scale = ns;
-        }
-        const float b = a * scale;
-        const float p = __fmul_rn(b, b), e = __fmaf_rn(b, b, -p);
-        const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-        c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z)), e));
-        s = t;
-    }
-    __device__ __forceinline__ double value() const {
-        const double u = 1.0 / (double)scale;   // exact
-        return ((double)s + (double)c) * u * u;
-    }
-};
-
-// The block's squared column norms into acc[0 .. dx): each lane's four columns
+// The block's squared column norms into acc[0 .. dx), in float64: each lane's four columns
 // c0 .. c0 + 3 of row group g (of ng), through part [ng][4 L].
-__device__ __forceinline__ void add_norms(const SumSq* q, bool act, int g, int ng, int c0, int dx, int L, double* part,
+__device__ __forceinline__ void add_norms(const double* q, bool act, int g, int ng, int c0, int dx, int L, double* part,
                                           double* __restrict__ acc) {
     if (act)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) part[g * 4 * L + c0 + k] = q[k].value();
+        for (int k = 0; k < 4; ++k) part[g * 4 * L + c0 + k] = q[k];
     __syncthreads();
     if ((int)threadIdx.x < dx) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -896,7 +868,7 @@ __global__ void __launch_bounds__(kPcolThreads, kPcolBlocks) k_pack_cols(const f
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane / L, k = lane - sub * L, c0 = 4 * k;
     const bool act = sub < G;
-    SumSq q[4];
+    double q[4] = {0.0, 0.0, 0.0, 0.0};
     const int64_t r0 = (int64_t)blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
     if (act)
         for (int64_t r = r0 + warp * G + sub; r < r1; r += ng) {
@@ -905,7 +877,7 @@ __global__ void __launch_bounds__(kPcolThreads, kPcolBlocks) k_pack_cols(const f
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 v[u] = c0 + u < dx ? src[c0 + u] : 0.f;
-                q[u].add(v[u]);
+                q[u] = fma((double)v[u], (double)v[u], q[u]);
             }
             xp[r * L + k] = make_float4(v[0], v[1], v[2], v[3]);
         }
@@ -924,9 +896,11 @@ __global__ void k_unpack_cols(const float4* __restrict__ yp, const int32_t* __re
 // y = A (x / ||x||) on the copy: L = ceil(dx / 4) lanes per row, a block taking
 // rows_per_block consecutive rows.  Each (row, column) sum is one fmaf chain
 // over the row's entries in order, then the column's scale.  Bound by the gathers
-// from L1 and L2.  250k rows, 21 columns: 126 -> 73 us a step; 128-thread blocks,
-// whose regions do not meet in L1, 95; padding the rows to whole 128-byte lines
-// made it 109; one block of 1024 per SM 81.
+// from L1 and L2, behind which the float64 sums of squares (units at a 64th of the
+// rate) are hidden: 67 us a step of 250k rows and 21 columns, where two float32 values
+// with their exact errors, of 46 bits, took 73 and three, of 53 bits, 79.  In node
+// order 126; the other forms with the two-value sums: 128-thread blocks, whose regions do
+// not meet in L1, 95; rows padded to whole 128-byte lines 109; one block of 1024 per SM 81.
 __global__ void __launch_bounds__(kPcolThreads, kPcolBlocks) k_spmv_pcols(const uint32_t* __restrict__ prp,
                                                              const int2* __restrict__ ent,
                                                              const float4* __restrict__ x, int64_t n, int dx,
@@ -939,7 +913,7 @@ __global__ void __launch_bounds__(kPcolThreads, kPcolBlocks) k_spmv_pcols(const 
     const int sub = lane / L, k = lane - sub * L, c0 = 4 * k;
     const bool act = sub < G;
     float sc[4];
-    SumSq q[4];
+    double q[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const double nn = (act && c0 + u < dx) ? n2_in[c0 + u] : 0.0;
@@ -967,10 +941,10 @@ __global__ void __launch_bounds__(kPcolThreads, kPcolBlocks) k_spmv_pcols(const 
                     }
             }
             a = make_float4(a.x * sc[0], a.y * sc[1], a.z * sc[2], a.w * sc[3]);
-            q[0].add(a.x);
-            q[1].add(a.y);
-            q[2].add(a.z);
-            q[3].add(a.w);
+            q[0] = fma((double)a.x, (double)a.x, q[0]);
+            q[1] = fma((double)a.y, (double)a.y, q[1]);
+            q[2] = fma((double)a.z, (double)a.z, q[2]);
+            q[3] = fma((double)a.w, (double)a.w, q[3]);
             y[r * L + k] = a;
         }
     add_norms(q, act, warp * G + sub, ng, c0, dx, L, part, n2_out);

@@ -172,3 +172,16 @@ def test_knn_time_with_far_points(kind):
     """A few points far from all others do not hold up the search of a hundred
     thousand (2490 and 431 ms where one thread walked all rings of cells)."""
     assert _knn_ms(ludvig.Scene.from_inputs(_scene_at(_far_points(kind, 100_000))), 16) <= 40.0
+
+
+@pytest.mark.parametrize("dx", [2, 5, 32])
+def test_column_norms_hold_beside_huge_and_tiny_columns(dx):
+    """Each column is scaled by its own norm, summed in float64: its result is that of
+    the column scaled by a power of two, bit for bit apart from the sums' order."""
+    s = inputs.scene_clusters(20_000, seed=5, n_clusters=6, sigma=0.1, extent=1.0)
+    g = ludvig.Graph(ludvig.Scene.from_inputs(s), 8, torch.ones((s.n, 4), device="cuda"), spatial_h=0.01)
+    x = torch.rand((s.n, dx), device="cuda", generator=torch.Generator("cuda").manual_seed(dx))
+    scale = torch.tensor([2.0 ** (((c * 37) % 120) - 60) for c in range(dx)], device="cuda")
+    a, b = g.diffuse(x, 3), g.diffuse(x * scale, 3)
+    assert rel_l2(b.cpu().numpy(), a.cpu().numpy()) <= 1e-6
+    assert torch.isfinite(b).all() and (b.norm(dim=0) > 0).all()
