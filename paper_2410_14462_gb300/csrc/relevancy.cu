@@ -13,14 +13,16 @@
 // float32 pairs of embeddings.  Every warp streams its own rows, in chunks of 12
 // channels by cp.async, the next one in flight while one is used; the blocks
 // are persistent, so the embeddings are normalised once per block.  Each dot
-// product is one fmaf chain over the channels in order, and so is the row's
-// squared norm.
+// product is one fmaf chain over the channels in order, the row's squared norm
+// two, over the even and the odd ones.
 //
 // Bound: the FMA pipe with the embeddings' shared-memory reads close behind (n d m
-// multiply-adds, m rounded up to a multiple of 4; the pipe is 0.53 busy).  500k x
-// 512 features, 21 queries and 4 phrases: 874 -> 465 us against tiles of 4 rows x 4
-// embeddings per thread, padded to 32.  Four rows per lane at 8 warps per SM, and
-// scalar instead of packed multiply-adds, measured 460 and 520 us.
+// multiply-adds, m rounded up to a multiple of 4).  500k x 512 features, 21 queries
+// and 4 phrases: 874 -> 465 us against tiles of 4 rows x 4 embeddings per thread, padded
+// to 32, and 412 with the norm's products in packed pairs behind a step's dots (before
+// them, or one by one between them, the accumulators spill: 478).  Four rows per lane at 8
+// warps per SM, and scalar instead of packed multiply-adds, measured 460 and 520 us
+// where this form took 465.
 #include <algorithm>
 
 #include "common.cuh"
@@ -83,10 +85,10 @@ __device__ __forceinline__ void relevancy_rows(const RelArgs& g, const float* sp
     __syncwarp();
     load_chunk(0);
     F2 acc[R][M / 2];
-    float nn[R];
+    F2 norm[R];
 #pragma unroll
     for (int a = 0; a < R; ++a) {
-        nn[a] = 0.f;
+        norm[a] = f2(0.f, 0.f);
 #pragma unroll
         for (int e = 0; e < M / 2; ++e) acc[a][e] = f2(0.f, 0.f);
     }
@@ -100,7 +102,9 @@ __device__ __forceinline__ void relevancy_rows(const RelArgs& g, const float* sp
         for (int c = 0; c < cw; c += 4) {
             float4 x[R];
 #pragma unroll
-            for (int a = 0; a < R; ++a) x[a] = *reinterpret_cast<const float4*>(st + a * (32 * kRelChunk) + c);
+            for (int a = 0; a < R; ++a) {
+                x[a] = *reinterpret_cast<const float4*>(st + a * (32 * kRelChunk) + c);
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float* pr = sphi + (size_t)(c0 + c + q) * M;
@@ -108,7 +112,6 @@ __device__ __forceinline__ void relevancy_rows(const RelArgs& g, const float* sp
 #pragma unroll
                 for (int a = 0; a < R; ++a) {
                     const float v = q == 0 ? x[a].x : q == 1 ? x[a].y : q == 2 ? x[a].z : x[a].w;
-                    nn[a] = fmaf(v, v, nn[a]);
                     xx[a] = f2(v, v);
                 }
 #pragma unroll
@@ -120,6 +123,11 @@ __device__ __forceinline__ void relevancy_rows(const RelArgs& g, const float* sp
                         acc[a][2 * e + 1] = f2_fma(xx[a], F2{p.y}, acc[a][2 * e + 1]);
                     }
                 }
+            }
+#pragma unroll
+            for (int a = 0; a < R; ++a) {
+                const F2 lo = f2(x[a].x, x[a].y), hi = f2(x[a].z, x[a].w);
+                norm[a] = f2_fma(hi, hi, f2_fma(lo, lo, norm[a]));
             }
         }
     }
@@ -135,8 +143,10 @@ __device__ __forceinline__ void relevancy_rows(const RelArgs& g, const float* sp
             s[2 * e] = v.x;
             s[2 * e + 1] = v.y;
         }
-        const float inv = nn[a] > 0.f ? 1.0f / sqrtf(nn[a]) : 0.f;
-        if (isfinite(nn[a])) {
+        const float2 halves = f2_get(norm[a]);
+        const float nn = halves.x + halves.y;
+        const float inv = nn > 0.f ? 1.0f / sqrtf(nn) : 0.f;
+        if (isfinite(nn)) {
             // 1 / (1 + exp(T inv (s_k - s_q))) falls with s_k: the largest phrase decides
             float top = -INFINITY;
 #pragma unroll
@@ -216,7 +226,7 @@ ludvig_status launch_relevancy(const float* f, int64_t n, int d, const float* ph
     LV_CUDA(cudaGetDevice(&dev));
     LV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // one block per SM, of as many warps as have room for their stage (at least
-    // 11: the embeddings take at most 160 KB)
+    // 8: the embeddings take at most 160 KB, a stage 8 KB)
     const size_t stage = sizeof(float) * rel_stage<M>(), embed = sizeof(float) * (size_t)((d + 3) & ~3) * M;
     const int nwarps = (int)std::min<size_t>(kRelWarps, (227 * 1024 - embed) / stage);
     const size_t smem = embed + nwarps * stage;

@@ -185,3 +185,16 @@ def test_column_norms_hold_beside_huge_and_tiny_columns(dx):
     a, b = g.diffuse(x, 3), g.diffuse(x * scale, 3)
     assert rel_l2(b.cpu().numpy(), a.cpu().numpy()) <= 1e-6
     assert torch.isfinite(b).all() and (b.norm(dim=0) > 0).all()
+
+
+def test_relevancy_norm_keeps_small_channels():
+    """One channel of 1 and 511 whose squares lie below half a unit of 1: of the two
+    chains that sum a row's squares one keeps its 256 small ones. What the other loses
+    (255 of 2^-25, 7.6e-6 of the norm, 3.8e-6 of its root) moves the score by at most
+    1.04e-6 at a logit of 1.54, its rounding by 2e-7; one chain would lose all, 2.06e-6."""
+    f = np.full((70, 512), 2.0 ** -12.5, np.float32)
+    f[:, 0] = 1.0
+    q, c = np.zeros((1, 512), np.float32), np.zeros((1, 512), np.float32)
+    q[0, 0], c[0, 1] = 1.0, 1.0
+    got = ludvig.relevancy(*(torch.from_numpy(a).cuda() for a in (f, q, c)), 1.54).cpu().numpy()
+    assert np.abs(got - oracle.relevancy(f, q, c, 1.54)).max() <= 1.3e-6
