@@ -1,0 +1,72 @@
+"""Groups of views and the forms of the weights pass: launches far above and below the
+few-tile limits give the same sums, packed jobs of uneven scenes share groups whose
+sorts run ahead, and a call that fails between its groups leaves nothing behind.
+Float32 sums of the same terms in another order: 1e-5 relative L2."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2410_14462_gb300 import inputs, ludvig
+from tests.gpu_util import device_features, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    from paper_2410_14462_gb300 import build
+    build.build()
+    ludvig.load()
+
+
+@pytest.fixture
+def option():
+    """Sets options for one test and puts them back."""
+    old = {}
+
+    def set_(name, value):
+        old.setdefault(name, ludvig.get_option(name))
+        ludvig.set_option(name, value)
+    yield set_
+    for name, value in old.items():
+        ludvig.set_option(name, value)
+
+
+def _same(got, ref):
+    assert (ref[1] > 0).any()
+    assert rel_l2(got[0].cpu().numpy(), ref[0].cpu().numpy()) <= 1e-5
+    assert rel_l2(got[1].cpu().numpy(), ref[1].cpu().numpy()) <= 1e-5
+
+
+# 9 views of 60 x 34 tiles: 18360 items in one group, then 2040 in each of nine
+@pytest.mark.parametrize("d,dtype,count", [(1, torch.float32, False), (4, torch.bfloat16, True), (27, torch.float32, False),
+                                           (40, torch.float32, True), (48, torch.bfloat16, False)])
+def test_many_and_few_tiles_agree(option, d, dtype, count):
+    wl = inputs.small_field_workload(n=20_000, views=9, d=d, width=955, height=539)
+    sc = ludvig.Scene.from_inputs(wl.scene)
+    F = device_features(wl, range(9), dtype=dtype)
+    option(ludvig.OPT_COUNT_NORMALISE, int(count))
+    one = ludvig.uplift(sc, wl.cams.params, 955, 539, F)
+    option(ludvig.OPT_GROUP_MB, 1)
+    _same(ludvig.uplift(sc, wl.cams.params, 955, 539, F), one)
+
+
+@pytest.mark.parametrize("d,dtype", [(3, torch.bfloat16), (40, torch.float32), (64, torch.bfloat16)])
+def test_packed_jobs_of_uneven_scenes(option, d, dtype):
+    option(ludvig.OPT_BATCH_TUNE, 0)
+    option(ludvig.OPT_GROUP_MB, 128)
+    jobs, ref = [], []
+    wls = [inputs.small_field_workload(n=n, views=v, d=d, width=157, height=93)
+           for n, v in ((300_000, 7), (20_000, 5), (150_000, 9), (70_000, 12))]
+    pool = torch.cat([device_features(wl, range(wl.cams.v), dtype=dtype) for wl in wls])   # (one class: views of one array)
+    at = 0
+    for wl in wls:
+        F = pool[at:at + wl.cams.v]
+        at += wl.cams.v
+        jobs.append((ludvig.Scene.from_inputs(wl.scene), wl.cams.params, 157, 93, F, None, None))
+        ref.append(ludvig.uplift(ludvig.Scene.from_inputs(wl.scene), wl.cams.params, 157, 93, F))
+    for _ in range(2):
+        for got, r in zip(ludvig.uplift_batch(jobs)[0], ref):
+            _same(got, r)
