@@ -1540,13 +1540,14 @@ ludvig_status enqueue_async(ludvig_scene* s, const std::vector<GroupViews>& grou
     LV_CUDA(cudaEventRecord(s->ev_call, st));
     LV_CUDA(cudaStreamWaitEvent(sf, s->ev_call, 0));
     LV_CUDA(cudaStreamWaitEvent(sa, s->ev_call, 0));
-    // on a failure, the projection of a group that will not run must not run on
-    // beside the next call
-    struct PreDrain {
+    // on a failure, nothing may run on that is not ordered on the caller's stream: the
+    // caller may use the outputs' memory again, and the next call this workspace
+    struct Drain {
         ludvig_scene* s;
-        bool armed = false;
-        ~PreDrain() {
-            if (armed) cudaStreamSynchronize(s->st_pre);
+        bool armed = true;
+        ~Drain() {
+            if (!armed) return;
+            for (cudaStream_t q : {s->st_pre, s->st_front, s->st_agg}) cudaStreamSynchronize(q);
         }
     } drain{s};
     for (size_t k = first; k < groups.size(); ++k) {
@@ -1564,17 +1565,16 @@ ludvig_status enqueue_async(ludvig_scene* s, const std::vector<GroupViews>& grou
         ccap->push_back(cc);
         if (k + 1 < groups.size()) {   // (enqueued behind this group's weights pass)
             FrontBufs b;
-            drain.armed = true;
             LV_CUDA(cudaStreamWaitEvent(s->st_pre, s->ev_sorted, 0));
             LV_TRY(project_and_sort(s, groups[k + 1], width, height, nullptr, s->st_pre, &b));
             LV_CUDA(cudaEventRecord(s->ev_pre, s->st_pre));
         }
     }
-    drain.armed = false;
     LV_CUDA(cudaEventRecord(s->ev_join[0], sf));
     LV_CUDA(cudaEventRecord(s->ev_join[1], sa));
     LV_CUDA(cudaStreamWaitEvent(st, s->ev_join[0], 0));
     LV_CUDA(cudaStreamWaitEvent(st, s->ev_join[1], 0));
+    drain.armed = false;
     return LUDVIG_OK;
 }
 

@@ -70,3 +70,32 @@ def test_packed_jobs_of_uneven_scenes(option, d, dtype):
     for _ in range(2):
         for got, r in zip(ludvig.uplift_batch(jobs)[0], ref):
             _same(got, r)
+
+
+@pytest.mark.parametrize("d,dtype", [(3, torch.bfloat16), (40, torch.float32), (100, torch.float32)])
+def test_failure_between_groups_leaves_nothing_running(option, d, dtype):
+    """An error that a launch check reports (injected on the host) while other groups'
+    work is queued: once it is raised, nothing of the call runs on but what is ordered
+    on the caller's stream, so that the caller may use the memory again."""
+    wl = inputs.small_field_workload(n=300_000, views=10, d=d, width=157, height=93)
+    sc = ludvig.Scene.from_inputs(wl.scene)
+    F = device_features(wl, range(10), dtype=dtype)
+    option(ludvig.OPT_GROUP_MB, 128)
+    ref = ludvig.uplift(sc, wl.cams.params, 157, 93, F)
+    out, beta = torch.empty_like(ref[0]), torch.empty_like(ref[1])
+    failed = 0
+    for k in (20, 33, 45, 52, 60, 71, 84, 97, 110, 125, 140):
+        torch.cuda._sleep(20_000_000)   # about 10 ms of SM clock, so that the queue is full when the call fails
+        ludvig.set_option(ludvig.OPT_FAULT_LAUNCH, k)
+        try:
+            ludvig.uplift(sc, wl.cams.params, 157, 93, F, out, beta)
+        except ludvig.LudvigError:
+            failed += 1
+            out.fill_(7.0)   # behind what the call put on this stream
+            beta.fill_(7.0)
+            torch.cuda.synchronize()
+            assert (out == 7.0).all() and (beta == 7.0).all(), k
+        finally:
+            ludvig.set_option(ludvig.OPT_FAULT_LAUNCH, 0)
+        _same(ludvig.uplift(sc, wl.cams.params, 157, 93, F, out, beta), ref)
+    assert failed >= 5
