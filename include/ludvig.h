@@ -49,7 +49,8 @@
  *    (ties: lower index first) alpha = min(0.99, o * exp(-0.5 d^T C d)); a
  *    Gaussian with alpha < 1/255 is skipped; the walk stops before the
  *    Gaussian that would take the transmittance below 1e-4;
- *    w = alpha * T.
+ *    w = alpha * T.  A Gaussian whose alpha is not a number at a pixel (its
+ *    opacity is a NaN) is skipped there.
  */
 #ifndef LUDVIG_H
 #define LUDVIG_H
@@ -76,7 +77,7 @@ typedef enum {
     LUDVIG_F32 = 0,              /* float32 features.  4 < d < 32, or 32 <= d <= 512 with
                                     d % 8 == 0: tensor-core aggregation with features and weights
                                     split into two bfloat16 terms each (float32-level accuracy);
-                                    d <= 4: the same weight terms summed in the compositing pass;
+                                    d <= 4: float32 weights summed in the compositing pass;
                                     otherwise, or with LUDVIG_OPT_F32_TENSOR_CORES = 0, CUDA-core
                                     FFMA */
     LUDVIG_BF16 = 1              /* bfloat16 features.  4 < d < 32, or 32 <= d <= 512 with
@@ -197,8 +198,8 @@ int64_t ludvig_scene_workspace_bytes(ludvig_scene_t scene);
  * sharding, checkpoint/resume).  Summation order on the GPU is not fixed
  * (atomics), so results are reproducible only to rounding.
  * Where the products run: d <= 4 in the compositing pass itself (each weight
- * row, split into bfloat16 terms as below, is dotted with the tile's features
- * on CUDA cores as it is made); 4 < d < 32, or 32 <= d <= 512 with d % 8 == 0,
+ * row, float32 or rounded to bfloat16 as the features are, is dotted with the
+ * tile's features on CUDA cores as it is made); 4 < d < 32, or 32 <= d <= 512 with d % 8 == 0,
  * on the tensor cores (4 < d < 32 on features the library zero-pads to 32
  * channels in its workspace), float32 features as split-bfloat16 terms
  * (float32-level accuracy; LUDVIG_OPT_F32_TENSOR_CORES = 0 moves them, and
@@ -206,8 +207,8 @@ int64_t ludvig_scene_workspace_bytes(ludvig_scene_t scene);
  * to bfloat16 for the product; any other d on CUDA cores with float32 weights.
  * Asynchronous: num/den are complete once ludvig_sync(scene) has returned
  * LUDVIG_OK (the views run in groups of up to 128; a group's projection, sorts
- * and weights overlap the previous group's products on two internal streams
- * that are joined back into `stream`). */
+ * and weights overlap the previous group's products on three internal streams
+ * that are joined back into `stream`; a call that fails waits for them). */
 ludvig_status ludvig_uplift_accumulate(ludvig_scene_t scene, const ludvig_camera* cams,
                                        int32_t n_views, int32_t width, int32_t height,
                                        const void* feats, int32_t dtype, int32_t d,
@@ -296,7 +297,7 @@ typedef struct {
  * (bound / 64 for float32: its weight rows grow with its pixels).  A class
  * that runs out of device memory is redone with half the bound (down to
  * 64 MiB).  The classes run one after another, largest first, on one
- * pooled context (its own workspace and two streams) driven by the calling
+ * pooled context (its own workspace and three streams) driven by the calling
  * thread; the other jobs run as ludvig_uplift calls on `slots` host threads
  * (the calling thread joins them after the classes) with pooled workspaces
  * lent to their scenes.  1 <= slots <=

@@ -1788,7 +1788,7 @@ __global__ void k_topfrac_mark(const uint32_t* __restrict__ vals, const float* _
 }
 
 // Reachability as bit sets (bit q = query column q): s_{t+1,i} = OR over the
-// row's edges with A_ij > 0 of s_t,j, one warp per row.
+// row's edges with A_ij > 0 of s_t,j.  The bits lie in the renumbered copy's order.
 __global__ void k_reach_init(const float* __restrict__ g0, const int32_t* __restrict__ inv, int64_t n, int dx,
                              uint32_t* __restrict__ s) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

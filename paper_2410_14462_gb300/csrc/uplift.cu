@@ -1264,7 +1264,7 @@ ludvig_status uplift_group(ludvig_scene* ctx, const GroupViews& g, int width, in
         // a few channels: the weights pass adds each row's W^T F and den into
         // the (padded) numerator itself; no weight rows, no aggregation
         int* cnt = nullptr;
-        LV_TRY(tc_weights_direct(fe.L, nv, width, height, fdt == LUDVIG_F32 ? 2 : 1, src.d, kPadD, f, fdt, av, s->ws,
+        LV_TRY(tc_weights_direct(fe.L, nv, width, height, fdt == LUDVIG_F32 ? 2 : 1, src.d, kPadD, f, av, s->ws,
                                  p, s->dstat, !ex.async, sf, &cnt));
         if (ex.async) {
             LV_CUDA(cudaMemcpyAsync(&ex.diag->chunks, cnt, sizeof(int), cudaMemcpyDeviceToDevice, sf));

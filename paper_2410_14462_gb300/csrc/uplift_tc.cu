@@ -10,9 +10,10 @@
 // the residuals are below 2^-16 relative).  den sums the same W terms, so each
 // f_i stays a convex combination of the features.
 //
-// Two kernels per chunk of views:
+// Two kernels per group of views:
 //
-//  k_weights (CUDA cores, one warp per (view, tile), see the kernel): walks the
+//  k_weights (CUDA cores, one warp per (view, tile), see the kernel; launches of
+//  few tiles take k_weights_block, eight warps per tile): walks the
 //  tile's depth-ordered list (float32 rules of Eq. 1: alpha, 1/255 skip, 1e-4
 //  stop) with two neighbouring pixels per lane in packed float32 arithmetic,
 //  and appends the Gaussians with a non-zero weight somewhere in the tile, as
@@ -98,7 +99,7 @@ struct WeightsArgs {
     int cap;
     float* chunk_den;       // [cap][128][NT]: each row's den, the sum of its weight terms, in term 0's
                             // slot (term 1's: 0); rewritten on a re-run
-    // direct accumulation (k_weights<NT, true>, few channels): each new row's
+    // direct accumulation (k_weights with DD > 0 channels): each new row's
     // sum_p w F[p, c] and its den go straight into the view's num and den
     // (atomic adds); no weight rows, chunks or plan are written
     int num_stride;         // floats per Gaussian in num
@@ -231,9 +232,9 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
     const uint32_t nb = (range.y - range.x + 31u) / 32u;
     float* const vnum = kDirect ? a.views.num[v] : nullptr;
     float* const vden = kDirect ? a.views.den[v] : nullptr;
-    // sum `i` of the kept rows over the lanes
     // byte of quadrant b's first pixel in a row
-    auto kQuadByte = [](int b) { return ((b >> 1) * 128 + (b & 1) * 8) * kPx; };
+    auto quad_byte = [](int b) { return ((b >> 1) * 128 + (b & 1) * 8) * kPx; };
+    // sum `i` of the kept rows over the lanes
     auto lane_sum = [&](int i) {
         const float* p = s_part + 33 * i;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -360,12 +361,12 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                             const __nv_bfloat162 h = __floats2bfloat162_rn(wx, wy);
                             const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
                             const F2 hf = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u));
-                            if (!kDirect) *reinterpret_cast<uint32_t*>(d1 + kQuadByte(b)) = hb;
+                            if (!kDirect) *reinterpret_cast<uint32_t*>(d1 + quad_byte(b)) = hb;
                             if (!kDirect && NT == 2) {   // w - h is exact
                                 const float2 res = f2_get(f2_fma(hf, f2(-1.f, -1.f), wv));
                                 const __nv_bfloat162 l = __floats2bfloat162_rn(res.x, res.y);
                                 const uint32_t lb = *reinterpret_cast<const uint32_t*>(&l);
-                                *reinterpret_cast<uint32_t*>(d2 + kQuadByte(b)) = lb;
+                                *reinterpret_cast<uint32_t*>(d2 + quad_byte(b)) = lb;
                                 if (!COUNT)
                                     den = f2_add(den, f2(__uint_as_float(lb << 16), __uint_as_float(lb & 0xffff0000u)));
                             }
@@ -385,8 +386,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
                             if (B[b] & bit) {
                                 finish(b, alpha(g, b));
                             } else if (!kDirect) {
-                                *reinterpret_cast<uint32_t*>(d1 + kQuadByte(b)) = 0u;
-                                if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + kQuadByte(b)) = 0u;
+                                *reinterpret_cast<uint32_t*>(d1 + quad_byte(b)) = 0u;
+                                if (NT == 2) *reinterpret_cast<uint32_t*>(d2 + quad_byte(b)) = 0u;
                             }
                         };
                         // side by side where all four are reached (independent chains)
@@ -1975,7 +1976,7 @@ void launch_weights_direct(const WeightsArgs& w, int d, int nitems, cudaStream_t
 }  // namespace
 
 ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int height, int NT, int d, int num_stride,
-                                const void* feats, int feat_dtype, const AggViews& av, Arena& ws, int parity,
+                                const void* feats, const AggViews& av, Arena& ws, int parity,
                                 int* status, bool checked, cudaStream_t st, int** counter) {
     if (!tc_direct_supported(d) || nv < 1 || nv > kMaxGroupViews) {
         set_error("direct accumulation takes 1 to %d channels and 1 to %d views", kDirectMaxD, kMaxGroupViews);
