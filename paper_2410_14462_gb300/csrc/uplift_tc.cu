@@ -106,6 +106,12 @@ struct WeightsArgs {
     const void* feats;      // [.., H, W, DD] float32 (NT = 2) or bfloat16, views at views.fview
     float2 one;             // {1, 1}: see f2_sum
     AggViews views;
+    // tiles that a warp hands over (see kHandover): item, entries walked, chunk being
+    // filled (-1: none yet) and its rows; the pixels' transmittances [..][256]
+    int4* rest;
+    float* rest_t;
+    int* rest_count;        // [0] handed over, [1] taken up in the second turn and later
+    uint32_t limit;         // the batches after which it does (none: all ones)
 };
 
 constexpr int kDirectMaxD = 4;
@@ -116,6 +122,19 @@ constexpr int kQuadItems = 152 * 16;
 // 1920 tiles 864 and 937 us, 2349 tiles 1011 and 1203; 2660 tiles equal, 3600 tiles 1051
 // and 1008.  (Evenly spread scenes cross earlier: 1920 tiles 672 and 664, 2349 771 and 709.)
 constexpr int kBlockItems = 152 * 16;
+
+// A tile whose pixels stay open over thousands of entries keeps one warp busy long after
+// all others have ended, most of all when it starts late.  In launches of up to two waves
+// of warps, which wait for such tiles, a warp hands its tile over after kHandover batches
+// of 32 entries to a second launch, where eight warps (rows) or four (direct) share what
+// is left.  16 views of 320x240, 1M Gaussians (4800 tiles), call of 40 float32 channels:
+// 6.9 ms without, 5.3, 5.3 and 5.2 with 32, 24 and 16 batches (5.2 with eight warps for
+// every tile); one channel 5.2, then 4.0, 3.9, 3.8; 9 views, 100k Gaussians 1.52, then
+// 1.42, 1.36, 1.31 (1.37).  Where no list is long the second launch costs 30 us (9 views of
+// an evenly spread scene, one channel, 0.69 -> 0.72 ms).  Larger launches have others to
+// run meanwhile: 60 views of 640x480 would go from 4.34 to 4.39 ms.
+constexpr uint32_t kHandover = 16;
+inline bool hands_over(int nitems, int sms) { return nitems < 2 * 28 * sms; }
 
 __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int rows, int next) {
     if (c >= 0 && c < a.cap) {
@@ -150,8 +169,9 @@ __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int ro
 // one block of 8 warps per tile that staged a batch's rows in shared memory; 48
 // views of 640x480, bfloat16 rows: 6.40 -> 3.37 ms; 60 views of 640x480, 3
 // channels direct: 6.81 -> 3.3 ms.
+// rest: the tile's place in a.rest, or -1 (all of its list).
 template <int NT, int DD, int NB, bool COUNT>
-__global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_constant__ WeightsArgs a) {
+__device__ __forceinline__ void weights_of_tile(const WeightsArgs& a, int item, int quad0, int rest) {
     constexpr bool kDirect = DD > 0;
     constexpr int kPx = 2;                        // bytes per pixel of a row
     constexpr int kVals = kDirect ? DD + 1 : 1;   // sums per row
@@ -163,9 +183,8 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
     __shared__ uint32_t s_gid[kRowBuf];
     const int lane = threadIdx.x;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    const int item = NB == 4 ? (int)blockIdx.x : (int)(blockIdx.x >> 2);
-    const int quad0 = NB == 4 ? 0 : (int)(blockIdx.x & 3u);
-    const uint2 range = a.ranges[item];
+    uint2 range = a.ranges[item];
+    if (rest >= 0) range.x += (uint32_t)a.rest[rest].y;
     if (range.x >= range.y) return;
     const int v = item / a.ntiles, tile = item - v * a.ntiles;
     const int tx = tile % a.TX, ty = tile / a.TX;
@@ -186,6 +205,19 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
 #pragma unroll
         for (int q = 0; q < 2; ++q)
             T[b][q] = px + 8 * (b & 1) + q < a.width && py + 8 * (b >> 1) < a.height ? 1.0f : 0.0f;
+    // this lane's first pixel of quadrant b in the tile
+    auto tile_pixel = [&](int b) {
+        const int q = NB == 4 ? b : quad0;
+        return ((lane >> 2) + 8 * (q >> 1)) * kTile + 8 * (q & 1) + 2 * (lane & 3);
+    };
+    if (rest >= 0) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const float2 t = *reinterpret_cast<const float2*>(a.rest_t + (size_t)rest * 256 + tile_pixel(b));
+            T[b][0] = t.x;
+            T[b][1] = t.y;
+        }
+    }
     F2 feat[kDirect ? DD : 1][NB];
     if constexpr (kDirect) {
 #pragma unroll
@@ -259,7 +291,12 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
         nbuf = 0;
     };
 
+    bool handed = false;
     for (uint32_t k = 0; k < nb && alive; ++k) {
+        if (NB == 4 && k == a.limit) {
+            handed = true;
+            break;
+        }
         const bool in = range.x + 32u * k + (uint32_t)lane < range.y;
         const uint32_t gid = __float_as_uint(rb.z);
         const uint32_t mask =
@@ -455,7 +492,35 @@ __global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_c
     if constexpr (kDirect) {
         if (nbuf > 0) flush_direct();
     } else {
-        if (lane == 0 && cur >= 0) finish_chunk(a, cur, local, -1);
+        if (!handed && lane == 0 && cur >= 0) finish_chunk(a, cur, local, -1);
+    }
+    if (NB == 4 && handed) {
+        int slot = 0;
+        if (lane == 0) {
+            slot = atomicAdd(a.rest_count, 1);
+            a.rest[slot] = make_int4(item, 32 * (int)a.limit, cur, cur < 0 ? 0 : local);
+        }
+        slot = __shfl_sync(kAll, slot, 0);
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+            *reinterpret_cast<float2*>(a.rest_t + (size_t)slot * 256 + tile_pixel(b)) = make_float2(T[b][0], T[b][1]);
+    }
+}
+
+// REST: the tiles handed over, taken in turn by any number of blocks.
+template <int NT, int DD, int NB, bool COUNT, bool REST>
+__global__ void __launch_bounds__(32, DD > 0 ? 24 : 28) k_weights(const __grid_constant__ WeightsArgs a) {
+    constexpr int kParts = 4 / NB;
+    if constexpr (REST) {
+        const int n = a.rest_count[0] * kParts;
+        for (int t = (int)blockIdx.x; t < n;) {
+            weights_of_tile<NT, DD, NB, COUNT>(a, a.rest[t / kParts].x, t % kParts, t / kParts);
+            __syncwarp();
+            if (threadIdx.x == 0) t = (int)gridDim.x + atomicAdd(a.rest_count + 1, 1);
+            t = __shfl_sync(0xffffffffu, t, 0);
+        }
+    } else {
+        weights_of_tile<NT, DD, NB, COUNT>(a, (int)blockIdx.x / kParts, (int)blockIdx.x % kParts, -1);
     }
 }
 
@@ -508,15 +573,17 @@ __device__ __forceinline__ float row_den(const uint32_t* wv, bool count_den, int
     return warp_sum(lane_den(wv, count_den, term));
 }
 
+// rest: the tile's place in a.rest, or -1 (all of its list).
 template <int NT, bool COUNT>
-__global__ void __launch_bounds__(256, 5) k_weights_block(const __grid_constant__ WeightsArgs a) {
-    __shared__ BlockSmem<NT> S;
+__device__ __forceinline__ void block_of_tile(const WeightsArgs& a, BlockSmem<NT>& S, int item, int rest) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    const int item = blockIdx.x;
     const int v = item / a.ntiles, tile = item - v * a.ntiles;
     const int tx = tile % a.TX, ty = tile / a.TX;
-    const uint2 range = a.ranges[item];
+    uint2 range = a.ranges[item];
+    int4 done_part = make_int4(item, 0, -1, 0);
+    if (rest >= 0) done_part = a.rest[rest];
+    range.x += (uint32_t)done_part.y;
     const uint32_t nb = (range.y - range.x + kTcBatch - 1) / kTcBatch;
     if (nb == 0) return;
     // warp w covers the 8x4 pixel block ((w & 1) * 8, (w >> 1) * 4) of the tile
@@ -528,7 +595,7 @@ __global__ void __launch_bounds__(256, 5) k_weights_block(const __grid_constant_
     if (tid == 0) {
         S.rowmask[0] = 0u;
         S.rowmask[1] = 0u;
-        S.cur_chunk = -1;
+        S.cur_chunk = done_part.z;
         S.cur_start = 0;
         S.next_chunk = -1;
     }
@@ -574,9 +641,10 @@ __global__ void __launch_bounds__(256, 5) k_weights_block(const __grid_constant_
         mask_batch(0);
     }
 
-    float T = 1.0f;
-    bool done = !(px < a.width && py < a.height);
-    int nrows = 0;   // rows of this tile written so far
+    float T = px < a.width && py < a.height ? 1.0f : 0.0f;
+    if (rest >= 0) T = a.rest_t[(size_t)rest * 256 + pix];
+    bool done = !(T > 0.f);
+    int nrows = done_part.w;   // rows of this tile from cur_chunk's first on
     int buf = 0;
     for (uint32_t k = 0; k < nb; ++k, buf ^= 1) {
         const uint32_t slot = k % kRing;
@@ -736,6 +804,24 @@ __global__ void __launch_bounds__(256, 5) k_weights_block(const __grid_constant_
             finish_chunk(a, cur, nrows - cstart, -1);
             finish_chunk(a, nxt, 0, -1);   // allocated, never used
         }
+    }
+}
+
+// REST: the tiles handed over, taken in turn by any number of blocks.
+template <int NT, bool COUNT, bool REST>
+__global__ void __launch_bounds__(256, 5) k_weights_block(const __grid_constant__ WeightsArgs a) {
+    __shared__ BlockSmem<NT> S;
+    if constexpr (REST) {
+        __shared__ int next;
+        const int n = a.rest_count[0];
+        for (int t = (int)blockIdx.x; t < n; t = next) {
+            __syncthreads();   // (the shared memory and `next` have been read)
+            block_of_tile<NT, COUNT>(a, S, a.rest[t].x, t);
+            if (threadIdx.x == 0) next = (int)gridDim.x + atomicAdd(a.rest_count + 1, 1);
+            __syncthreads();
+        }
+    } else {
+        block_of_tile<NT, COUNT>(a, S, (int)blockIdx.x, -1);
     }
 }
 
@@ -1826,11 +1912,21 @@ const char* const kWsCounter[2] = {"tc.counter.0", "tc.counter.1"};
 const char* const kWsPlanOff[2] = {"tc.plan_off.0", "tc.plan_off.1"};
 const char* const kWsPlan[2] = {"tc.plan.0", "tc.plan.1"};
 
+namespace {
+// The tiles that a launch of nitems may hand over.
+ludvig_status get_rest(Arena& ws, int nitems, int sms, WeightsArgs* w) {
+    w->limit = hands_over(nitems, sms) ? kHandover : 0xffffffffu;
+    if (!hands_over(nitems, sms)) return LUDVIG_OK;
+    LV_TRY(ws.get("tc.rest", (size_t)nitems, &w->rest));
+    return ws.get("tc.rest_t", (size_t)nitems * 256, &w->rest_t);
+}
+}  // namespace
+
 ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets) {
     cap = std::max<int64_t>(cap, 3 * (int64_t)nitems);
     for (int p = 0; p < sets; ++p) {
         void* q;
-        LV_TRY(ws.get(kWsCounter[p], sizeof(int), &q));
+        LV_TRY(ws.get(kWsCounter[p], 3 * sizeof(int), &q));
         LV_TRY(ws.get(kWsFirst[p], sizeof(int) * (size_t)nitems, &q));
         LV_TRY(ws.get(kWsW1[p], (size_t)cap * kChunkBytes, &q));
         if (NT == 2) LV_TRY(ws.get(kWsW2[p], (size_t)cap * kChunkBytes, &q));
@@ -1841,17 +1937,28 @@ ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets) {
         LV_TRY(ws.get(kWsPlanOff[p], sizeof(uint32_t) * ((size_t)nitems + 1), &q));
         LV_TRY(ws.get(kWsPlan[p], sizeof(int2) * (size_t)cap, &q));
     }
-    return LUDVIG_OK;
+    int sms = 0;
+    LV_TRY(sm_count(&sms));
+    WeightsArgs w;
+    return get_rest(ws, nitems, sms, &w);
 }
 
 namespace {
-template <int NT>
-void launch_weight_rows(const WeightsArgs& w, int nitems, cudaStream_t st) {
-    const bool count = option_count_normalise();
-    if (nitems < kBlockItems)
-        count ? k_weights_block<NT, true><<<nitems, 256, 0, st>>>(w) : k_weights_block<NT, false><<<nitems, 256, 0, st>>>(w);
-    else
-        count ? k_weights<NT, 0, 4, true><<<nitems, 32, 0, st>>>(w) : k_weights<NT, 0, 4, false><<<nitems, 32, 0, st>>>(w);
+// (The second launch as wide as the GPU: it finds out on the device how many tiles
+// there are for it, often none.)
+template <int NT, bool COUNT>
+ludvig_status launch_weight_rows(const WeightsArgs& w, int nitems, int sms, cudaStream_t st) {
+    if (nitems < kBlockItems) {
+        k_weights_block<NT, COUNT, false><<<nitems, 256, 0, st>>>(w);
+    } else {
+        k_weights<NT, 0, 4, COUNT, false><<<nitems, 32, 0, st>>>(w);
+        if (hands_over(nitems, sms)) {
+            LV_LAUNCH();
+            k_weights_block<NT, COUNT, true><<<std::min(nitems, 5 * sms), 256, 0, st>>>(w);
+        }
+    }
+    LV_LAUNCH();
+    return LUDVIG_OK;
 }
 }  // namespace
 
@@ -1861,7 +1968,9 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
     const int TX = (width + kTile - 1) / kTile, TY = (height + kTile - 1) / kTile;
     const int nitems = nv * TX * TY;
     TileWeights t;
-    LV_TRY(ws.get(kWsCounter[p], 1, &t.counter));
+    int sms = 0;
+    LV_TRY(sm_count(&sms));
+    LV_TRY(ws.get(kWsCounter[p], 3, &t.counter));   // [1], [2]: tiles handed over, and taken up
     LV_TRY(ws.get(kWsFirst[p], (size_t)nitems, &t.ifirst));
     int* host = nullptr;   // [0] chunks used, [1] status
     if (checked) {
@@ -1881,9 +1990,11 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         LV_TRY(ws.get(kWsRows[p], (size_t)cap, &t.crows));
         LV_TRY(ws.get(kWsNext[p], (size_t)cap, &t.cnext));
         LV_TRY(ws.get(kWsDen[p], (size_t)cap * kCRows * NT, &t.cden));
-        LV_CUDA(cudaMemsetAsync(t.counter, 0, sizeof(int), st));
+        LV_CUDA(cudaMemsetAsync(t.counter, 0, 3 * sizeof(int), st));
         LV_CUDA(cudaMemsetAsync(t.ifirst, 0xff, sizeof(int) * (size_t)nitems, st));
         WeightsArgs w{};
+        LV_TRY(get_rest(ws, nitems, sms, &w));
+        w.rest_count = t.counter + 1;
         w.rank = L.rank;
         w.srec = L.srec;
         w.npad = L.npad;
@@ -1903,11 +2014,10 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
         w.chunk_den = t.cden;
         w.one = make_float2(1.f, 1.f);
         const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
-        if (NT == 2)
-            launch_weight_rows<2>(w, nitems, st);
+        if (option_count_normalise())
+            LV_TRY((NT == 2 ? launch_weight_rows<2, true> : launch_weight_rows<1, true>)(w, nitems, sms, st));
         else
-            launch_weight_rows<1>(w, nitems, st);
-        LV_LAUNCH();
+            LV_TRY((NT == 2 ? launch_weight_rows<2, false> : launch_weight_rows<1, false>)(w, nitems, sms, st));
         trace_end(tslot, st);
         if (!checked) break;
         LV_CUDA(cudaMemcpyAsync(host, t.counter, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1950,28 +2060,33 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
 bool tc_direct_supported(int d) { return d >= 1 && d <= kDirectMaxD; }
 
 namespace {
-template <int NT, int NB, bool COUNT>
-void launch_weights_direct_nb(const WeightsArgs& w, int d, int nitems, cudaStream_t st) {
-    const unsigned grid = (unsigned)nitems * (4 / NB);
-    switch (d) {
-        case 1: k_weights<NT, 1, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
-        case 2: k_weights<NT, 2, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
-        case 3: k_weights<NT, 3, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
-        default: k_weights<NT, 4, NB, COUNT><<<grid, 32, 0, st>>>(w); break;
-    }
-}
-
-template <int NT>
-void launch_weights_direct(const WeightsArgs& w, int d, int nitems, cudaStream_t st) {
+template <int NT, int DD, bool COUNT>
+ludvig_status launch_weights_direct(const WeightsArgs& w, int nitems, int sms, cudaStream_t st) {
     // Whole tiles per warp, or, when the tiles would not give every scheduler
     // four warps, one quadrant per warp: a quadrant's rows cost the lane sums of
     // a whole row, but the longest tile's chain is a quarter (8 views of 128x128,
     // 512 tiles: 470 us by tiles, 182 by quadrants; 2048 tiles: 590 and 400)
-    const bool quads = nitems < kQuadItems;
-    if (option_count_normalise())
-        quads ? launch_weights_direct_nb<NT, 1, true>(w, d, nitems, st) : launch_weights_direct_nb<NT, 4, true>(w, d, nitems, st);
-    else
-        quads ? launch_weights_direct_nb<NT, 1, false>(w, d, nitems, st) : launch_weights_direct_nb<NT, 4, false>(w, d, nitems, st);
+    if (nitems < kQuadItems) {
+        k_weights<NT, DD, 1, COUNT, false><<<4 * nitems, 32, 0, st>>>(w);
+    } else {
+        k_weights<NT, DD, 4, COUNT, false><<<nitems, 32, 0, st>>>(w);
+        if (hands_over(nitems, sms)) {
+            LV_LAUNCH();
+            k_weights<NT, DD, 1, COUNT, true><<<std::min(4 * nitems, 24 * sms), 32, 0, st>>>(w);
+        }
+    }
+    LV_LAUNCH();
+    return LUDVIG_OK;
+}
+
+template <int NT, bool COUNT>
+ludvig_status launch_weights_direct(const WeightsArgs& w, int d, int nitems, int sms, cudaStream_t st) {
+    switch (d) {
+        case 1: return launch_weights_direct<NT, 1, COUNT>(w, nitems, sms, st);
+        case 2: return launch_weights_direct<NT, 2, COUNT>(w, nitems, sms, st);
+        case 3: return launch_weights_direct<NT, 3, COUNT>(w, nitems, sms, st);
+        default: return launch_weights_direct<NT, 4, COUNT>(w, nitems, sms, st);
+    }
 }
 }  // namespace
 
@@ -1986,9 +2101,13 @@ ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int heig
     const int TX = (width + kTile - 1) / kTile, TY = (height + kTile - 1) / kTile;
     const int nitems = nv * TX * TY;
     int* cnt;
-    LV_TRY(ws.get(kWsCounter[p], 1, &cnt));
-    LV_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int), st));
+    int sms = 0;
+    LV_TRY(sm_count(&sms));
+    LV_TRY(ws.get(kWsCounter[p], 3, &cnt));   // [1], [2]: tiles handed over, and taken up
+    LV_CUDA(cudaMemsetAsync(cnt, 0, 3 * sizeof(int), st));
     WeightsArgs w{};
+    LV_TRY(get_rest(ws, nitems, sms, &w));
+    w.rest_count = cnt + 1;
     w.rank = L.rank;
     w.srec = L.srec;
     w.npad = L.npad;
@@ -2003,11 +2122,10 @@ ludvig_status tc_weights_direct(const GroupLists& L, int nv, int width, int heig
     w.feats = feats;
     w.views = av;
     const int tslot = trace_on() ? trace_begin(LUDVIG_STAGE_WEIGHTS, st) : -1;
-    if (NT == 2)
-        launch_weights_direct<2>(w, d, nitems, st);
+    if (option_count_normalise())
+        LV_TRY((NT == 2 ? launch_weights_direct<2, true> : launch_weights_direct<1, true>)(w, d, nitems, sms, st));
     else
-        launch_weights_direct<1>(w, d, nitems, st);
-    LV_LAUNCH();
+        LV_TRY((NT == 2 ? launch_weights_direct<2, false> : launch_weights_direct<1, false>)(w, d, nitems, sms, st));
     trace_end(tslot, st);
     if (checked) {
         void* hp;

@@ -53,6 +53,36 @@ def test_many_and_few_tiles_agree(option, d, dtype, count):
     _same(ludvig.uplift(sc, wl.cams.params, 955, 539, F), one)
 
 
+def _faint_slab(n=180_000, seed=11):
+    """Faint Gaussians so dense that pixels stay open over hundreds of contributors."""
+    rng = np.random.default_rng(seed)
+    q = rng.normal(size=(n, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    return inputs.Scene((rng.uniform(-0.6, 0.6, size=(n, 3)) * [1.0, 1.0, 0.3]).astype(np.float32),
+                        np.full((n, 3), 0.03, np.float32), q.astype(np.float32), np.full(n, 0.012, np.float32))
+
+
+# 9 views of 20 x 15 tiles: 2700 items, whose long lists are handed over, then 300 in each of nine
+@pytest.mark.parametrize("d,dtype", [(1, torch.float32), (3, torch.bfloat16), (4, torch.float32), (40, torch.float32),
+                                     (48, torch.bfloat16)])
+@pytest.mark.parametrize("count", [False, True])
+def test_long_lists_handed_over(option, d, dtype, count):
+    scene = _faint_slab()
+    cams = inputs.cameras_orbit(9, 1.6, 315, 235, 250.0, hemisphere=True)
+    sc = ludvig.Scene.from_inputs(scene)
+    _, contributors = ludvig.debug_transmittance(sc, cams.params[0], 315, 235)
+    open_late = (contributors > 512).float().mean().item()
+    assert 0.05 < open_late   # more entries than a warp walks by itself
+    F = torch.rand((9, 235, 315, d), device="cuda", generator=torch.Generator("cuda").manual_seed(d)).to(dtype)
+    option(ludvig.OPT_COUNT_NORMALISE, int(count))
+    one = ludvig.uplift(sc, cams.params, 315, 235, F)
+    option(ludvig.OPT_GROUP_MB, 1)
+    few = ludvig.uplift(sc, cams.params, 315, 235, F)
+    _same(one, few)
+    if count:
+        assert torch.equal(one[1], few[1])
+
+
 @pytest.mark.parametrize("d,dtype", [(3, torch.bfloat16), (40, torch.float32), (64, torch.bfloat16)])
 def test_packed_jobs_of_uneven_scenes(option, d, dtype):
     option(ludvig.OPT_BATCH_TUNE, 0)
