@@ -115,13 +115,15 @@ struct WeightsArgs {
 };
 
 constexpr int kDirectMaxD = 4;
-constexpr int kQuadItems = 152 * 16;
-// Below: weight rows by blocks of 8 warps per tile.  With few tiles the longest list
-// sets the time, and eight warps share it; from about 16 tiles an SM the warps of whole
-// tiles fill it.  Blocks against warps, uplifts of 64 channels, 300k clustered Gaussians:
-// 1920 tiles 864 and 937 us, 2349 tiles 1011 and 1203; 2660 tiles equal, 3600 tiles 1051
-// and 1008.  (Evenly spread scenes cross earlier: 1920 tiles 672 and 664, 2349 771 and 709.)
-constexpr int kBlockItems = 152 * 16;
+// Tiles an SM, below which a launch has few.  Few-channel sums then go by quadrants (see
+// launch_weights_direct), weight rows by blocks of 8 warps per tile: with few tiles the
+// longest list sets the time, and eight warps share it; from about 16 tiles an SM the
+// warps of whole tiles fill it.  Blocks against warps, uplifts of 64 channels, 300k
+// clustered Gaussians: 1920 tiles 864 and 937 us, 2349 tiles 1011 and 1203 (evenly spread,
+// 672 and 664, 771 and 709); above, warps that hand long lists over (kHandover) are ahead:
+// 2700 tiles 1706 and 1590, 3600 tiles 1950 and 1827 (evenly spread, 979 and 926, 1142 and
+// 1038).
+constexpr int kFewTiles = 16;
 
 // A tile whose pixels stay open over thousands of entries keeps one warp busy long after
 // all others have ended, most of all when it starts late.  In launches of up to two waves
@@ -1948,7 +1950,7 @@ namespace {
 // there are for it, often none.)
 template <int NT, bool COUNT>
 ludvig_status launch_weight_rows(const WeightsArgs& w, int nitems, int sms, cudaStream_t st) {
-    if (nitems < kBlockItems) {
+    if (nitems < kFewTiles * sms) {
         k_weights_block<NT, COUNT, false><<<nitems, 256, 0, st>>>(w);
     } else {
         k_weights<NT, 0, 4, COUNT, false><<<nitems, 32, 0, st>>>(w);
@@ -2066,7 +2068,7 @@ ludvig_status launch_weights_direct(const WeightsArgs& w, int nitems, int sms, c
     // four warps, one quadrant per warp: a quadrant's rows cost the lane sums of
     // a whole row, but the longest tile's chain is a quarter (8 views of 128x128,
     // 512 tiles: 470 us by tiles, 182 by quadrants; 2048 tiles: 590 and 400)
-    if (nitems < kQuadItems) {
+    if (nitems < kFewTiles * sms) {
         k_weights<NT, DD, 1, COUNT, false><<<4 * nitems, 32, 0, st>>>(w);
     } else {
         k_weights<NT, DD, 4, COUNT, false><<<nitems, 32, 0, st>>>(w);

@@ -129,3 +129,21 @@ def test_failure_between_groups_leaves_nothing_running(option, d, dtype):
             ludvig.set_option(ludvig.OPT_FAULT_LAUNCH, 0)
         _same(ludvig.uplift(sc, wl.cams.params, 157, 93, F, out, beta), ref)
     assert failed >= 5
+
+
+@pytest.mark.parametrize("d,dtype", [(3, torch.float32), (40, torch.float32), (48, torch.bfloat16), (100, torch.float32),
+                                     (101, torch.bfloat16)])
+def test_a_call_that_outgrows_the_workspace_is_redone(d, dtype):
+    """A far view sizes the workspace; near ones, in an asynchronous call, need many times
+    its pairs and weight rows, with tiles handed over while the rows' capacity is exceeded."""
+    scene = _faint_slab()
+    far = inputs.cameras_orbit(1, 60.0, 16, 16, 60.0, hemisphere=True)
+    near = inputs.cameras_orbit(9, 1.6, 315, 235, 250.0, hemisphere=True)
+    F = torch.rand((9, 235, 315, d), device="cuda", generator=torch.Generator("cuda").manual_seed(d)).to(dtype)
+    ref = ludvig.uplift(ludvig.Scene.from_inputs(scene), near.params, 315, 235, F)
+    sc = ludvig.Scene.from_inputs(scene)
+    ludvig.uplift(sc, far.params, 16, 16, F[:1, :16, :16].contiguous())
+    small = sc.workspace_bytes()
+    _same(ludvig.uplift(sc, near.params, 315, 235, F), ref)
+    assert sc.workspace_bytes() > small
+    _same(ludvig.uplift(sc, near.params, 315, 235, F), ref)
