@@ -206,8 +206,10 @@ __global__ void __launch_bounds__(32 * kRelWarps, 1) k_relevancy(const RelArgs g
     }
     __syncthreads();
     // this warp's rows, 32 R at a time and what is left in halves (equal shares:
-    // whole groups alone would leave most warps idle in the last round)
-    int64_t r0 = ((int64_t)blockIdx.x * nwarps + warp) * rows_per_warp;
+    // whole groups alone would leave most warps idle in the last round), the shares
+    // dealt to the blocks in turn, so that few rows spread over all SMs: 5000 x 512, 25
+    // embeddings 125 -> 74 us (87 with blocks of 128 rows)
+    int64_t r0 = ((int64_t)warp * gridDim.x + blockIdx.x) * rows_per_warp;
     const int64_t r1 = min(g.n, r0 + rows_per_warp);
     constexpr int R = rel_rows(M);
     for (; r1 - r0 > 32 * (R - 1); r0 += 32 * R) relevancy_rows<M, R>(g, sphi, stage, r0);
@@ -232,7 +234,7 @@ ludvig_status launch_relevancy(const float* f, int64_t n, int d, const float* ph
     const size_t smem = embed + nwarps * stage;
     const int64_t rpw = std::max<int64_t>(32, round_up(ceil_div(n, (int64_t)sms * nwarps), 32));
     RelArgs g{f, n, d, nq, m, d % 4 == 0 && (reinterpret_cast<uintptr_t>(f) & 15) == 0, T, r};
-    k_relevancy<M><<<(unsigned)ceil_div(n, rpw * nwarps), 32 * nwarps, smem, st>>>(g, phi, rpw);
+    k_relevancy<M><<<(unsigned)std::min<int64_t>(sms, ceil_div(n, rpw)), 32 * nwarps, smem, st>>>(g, phi, rpw);
     LV_LAUNCH();
     return LUDVIG_OK;
 }
