@@ -530,7 +530,8 @@ ludvig_status ludvig_graph_export(ludvig_graph_t graph, int64_t* row_ptr, int32_
  * (32-row slices, column-major) that the first call after the graph's values
  * change builds in the graph's workspace; that call synchronises `stream`
  * once.  More columns run on a renumbered row copy, built the same way (without
- * a synchronisation). */
+ * a synchronisation) once the calls since the values changed have taken four
+ * steps. */
 ludvig_status ludvig_diffuse(ludvig_graph_t graph, const float* x0, int32_t dx, int32_t iters,
                              float* out, void* stream);
 

@@ -188,6 +188,8 @@ struct ludvig_graph {
     int sell_version = -1;        // val_version of the sliced copy in ws ("sell.*"), -1: none
     int64_t sell_slices = 0;
     int pcsr_version = -1;        // val_version of the renumbered row copy in ws ("pcsr.*"), -1: none
+    int64_t pcsr_steps = 0;       // steps taken without that copy since the values last changed
+    int pcsr_steps_version = -1;  // val_version they belong to
     int32_t* perm = nullptr;      // [n] node at position r of the centres' Morton order (null: identity)
     int32_t* inv = nullptr;       // [n] position of each node in that order
     ludvig::Arena ws;

@@ -1470,6 +1470,24 @@ ludvig_status ensure_pcsr(ludvig_graph* g, cudaStream_t st, uint32_t** prp, int2
     return LUDVIG_OK;
 }
 
+// Whether a call of `steps` steps of the given weight runs on the row copy: when the
+// copy is there, or once the steps taken without it since the values changed have cost
+// what building it costs (about 100 us: four diffusion steps or 32 reach steps).  So a
+// single short call does not pay for the copy (one diffusion step of 2 columns on 20k
+// nodes 104 us, 214 with it; one reach step 66 and 164; ten on 300k 400 and 437), and many
+// short calls pay for it once.
+constexpr int64_t kCopySteps = 32, kDiffuseWeight = 8, kReachWeight = 1;
+
+bool use_row_copy(ludvig_graph* g, int64_t steps, int64_t weight) {
+    if (g->pcsr_version == g->val_version) return true;
+    if (g->pcsr_steps_version != g->val_version) {
+        g->pcsr_steps = 0;
+        g->pcsr_steps_version = g->val_version;
+    }
+    g->pcsr_steps += std::min(steps, kCopySteps) * weight;
+    return g->pcsr_steps >= kCopySteps;
+}
+
 // ludvig_diffuse for two columns or more.
 ludvig_status diffuse_cols(ludvig_graph* g, const float* x0, int dx, int iters, float* out, double* n2, int sms,
                            cudaStream_t st) {
@@ -1523,19 +1541,19 @@ extern "C" ludvig_status ludvig_diffuse(ludvig_graph_t g, const float* x0, int32
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (dx > 1) return diffuse_cols(g, x0, dx, iters, out, n2, sms, st);
+    if (dx > 1 && use_row_copy(g, iters, kDiffuseWeight)) return diffuse_cols(g, x0, dx, iters, out, n2, sms, st);
     float* tmp;
-    LV_TRY(g->ws.get("d.tmp", (size_t)n, &tmp));
+    LV_TRY(g->ws.get("d.tmp", (size_t)n * dx, &tmp));
     // ping-pong so that the last step writes `out`
     float* bufs[2] = {(iters % 2 == 1) ? out : tmp, (iters % 2 == 1) ? tmp : out};
-    k_colnorm2<<<(unsigned)std::min<int64_t>(592, ceil_div(n, 256)), 256, 0, st>>>(x0, n, 1, n2);
+    k_colnorm2<<<(unsigned)std::min<int64_t>(592, ceil_div(n, 256)), 256, 0, st>>>(x0, n, dx, n2);
     LV_LAUNCH();
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * 8, ceil_div(n, 32)));
     bool sell = false;
     uint32_t* soff = nullptr;
     int32_t* scol = nullptr;
     float* sval = nullptr;
-    LV_TRY(ensure_sell(g, st, &sell, &soff, &scol, &sval));
+    if (dx == 1) LV_TRY(ensure_sell(g, st, &sell, &soff, &scol, &sval));
     // the renumbered sliced copy works on the permuted vector: x0 gathered in,
     // the last step's vector scattered back to out
     const bool permuted = sell && g->perm;
@@ -1551,6 +1569,9 @@ extern "C" ludvig_status ludvig_diffuse(ludvig_graph_t g, const float* x0, int32
         float* y = permuted ? ((t & 1) ? pa : pb) : bufs[t & 1];
         if (sell)
             k_spmv_sell<<<blocks, 256, 0, st>>>(soff, scol, sval, xin, n, g->sell_slices, n2 + 32 * t, y,
+                                                n2 + 32 * (t + 1));
+        else if (dx > 1)
+            k_spmv_cols<<<blocks, 256, 0, st>>>(g->row_ptr, g->col, g->val, xin, n, dx, n2 + 32 * t, y,
                                                 n2 + 32 * (t + 1));
         else
             k_spmv_scaled<8><<<blocks, 256, 0, st>>>(g->row_ptr, g->col, g->val, xin, n, 1, n2 + 32 * t, y,
@@ -1788,7 +1809,7 @@ __global__ void k_topfrac_mark(const uint32_t* __restrict__ vals, const float* _
 }
 
 // Reachability as bit sets (bit q = query column q): s_{t+1,i} = OR over the
-// row's edges with A_ij > 0 of s_t,j.  The bits lie in the renumbered copy's order.
+// row's edges with A_ij > 0 of s_t,j.
 __global__ void k_reach_init(const float* __restrict__ g0, const int32_t* __restrict__ inv, int64_t n, int dx,
                              uint32_t* __restrict__ s) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1819,6 +1840,22 @@ __global__ void __launch_bounds__(256) k_reach_step(const uint32_t* __restrict__
     b |= __shfl_xor_sync(0xffffffffu, b, 1);
     b |= __shfl_xor_sync(0xffffffffu, b, 2);
     if (r < n && sub == 0) s2[r] = b;
+}
+
+// The same on the CSR, eight lanes per row (a row holds k to 2k entries), for few steps
+// (see use_row_copy).
+__global__ void __launch_bounds__(256) k_reach_step_csr(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                                        const float* __restrict__ val, const uint32_t* __restrict__ s,
+                                                        int64_t n, uint32_t* __restrict__ s2) {
+    const int sub = threadIdx.x & 7;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    uint32_t b = 0u;
+    if (i < n)
+        for (int64_t e = rp[i] + sub, e1 = rp[i + 1]; e < e1; e += 8)
+            if (val[e] > 0.f) b |= s[col[e]];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) b |= __shfl_xor_sync(0xffffffffu, b, o);
+    if (i < n && sub == 0) s2[i] = b;
 }
 
 __global__ void k_reach_out(const uint32_t* __restrict__ s, const int32_t* __restrict__ inv,
@@ -1992,17 +2029,22 @@ extern "C" ludvig_status ludvig_reach_weight(ludvig_graph_t graph, const float* 
     LV_TRY(graph->ws.get("reach.s0", (size_t)n, &s0));
     LV_TRY(graph->ws.get("reach.s1", (size_t)n, &s1));
     StageScope scope(LUDVIG_STAGE_DIFFUSE, st);
+    const bool copy = use_row_copy(graph, steps, kReachWeight);
+    const int32_t* order = copy ? graph->inv : nullptr;   // the bits lie in the copy's order, or in the nodes'
     uint32_t* prp;
     int2* ent;
-    LV_TRY(ensure_pcsr(graph, st, &prp, &ent));
-    k_reach_init<<<grid_for(n, 256), 256, 0, st>>>(g0, graph->inv, n, dx, s0);
+    if (copy) LV_TRY(ensure_pcsr(graph, st, &prp, &ent));
+    k_reach_init<<<grid_for(n, 256), 256, 0, st>>>(g0, order, n, dx, s0);
     LV_LAUNCH();
     for (int t = 0; t < steps; ++t) {
-        k_reach_step<<<grid_for(n * 4, 256), 256, 0, st>>>(prp, ent, s0, n, s1);
+        if (copy)
+            k_reach_step<<<grid_for(n * 4, 256), 256, 0, st>>>(prp, ent, s0, n, s1);
+        else
+            k_reach_step_csr<<<grid_for(n * 8, 256), 256, 0, st>>>(graph->row_ptr, graph->col, graph->val, s0, n, s1);
         LV_LAUNCH();
         std::swap(s0, s1);
     }
-    k_reach_out<<<grid_for(n * dx, 256), 256, 0, st>>>(s0, graph->inv, unary, n, dx, h);
+    k_reach_out<<<grid_for(n * dx, 256), 256, 0, st>>>(s0, order, unary, n, dx, h);
     LV_LAUNCH();
     return LUDVIG_OK;
 }
