@@ -132,6 +132,9 @@ __global__ void k_gather_sorted(const float* __restrict__ x, const uint32_t* __r
 // z and y faces, one cell at either end elsewhere).  Bound by instruction issue
 // (a warp inserts whenever one of its lanes does).  1M clustered centres, k = 16:
 // 3.54 -> 2.3 ms with smaller cells, runs of cells and 64-bit (distance, index) keys.
+// (0: no bound; one block per SM as the bound takes more registers and 0.2 ms more.)
+// Four blocks per SM for K = 32 (the compiler takes three otherwise): 100k clustered
+// centres, k = 32, 1.21 -> 1.11 ms.
 template <int K>
 __device__ __forceinline__ void knn_insert(uint64_t (&best)[K], uint64_t key) {
 #pragma unroll
@@ -143,7 +146,7 @@ __device__ __forceinline__ void knn_insert(uint64_t (&best)[K], uint64_t key) {
 }
 
 template <int K>
-__global__ void __launch_bounds__(128) k_knn(const float4* __restrict__ pts, int64_t n, Grid gr,
+__global__ void __launch_bounds__(128, K <= 16 ? 0 : K <= 32 ? 4 : 2) k_knn(const float4* __restrict__ pts, int64_t n, Grid gr,
                                              const uint32_t* __restrict__ start, int k,
                                              int32_t* __restrict__ out, uint32_t* __restrict__ far,
                                              uint32_t* __restrict__ nfar) {
