@@ -19,13 +19,11 @@ namespace ludvig {
 
 namespace {
 
-// Both passes take a view's elements in pieces of kPieces x 256 groups of four
-// (float32) or eight (bfloat16): 16-byte loads, kPieces of them in flight per
-// thread.  A view that does not start on a 16-byte boundary (or whose codes do
-// not start on one of a group's size), and the end of a view, go element by
-// element.
-constexpr int kPieces = 4;
-
+// Both passes take a view's elements in pieces of P x 256 groups of four (float32)
+// or eight (bfloat16): 16-byte loads, P = 4 of them in flight per thread, or one where
+// the views are too small to give every SM a few pieces of four.  A view that does not
+// start on a 16-byte boundary (or whose codes do not start on one of a group's size), and
+// the end of a view, go element by element, four at a time.
 template <class T>
 struct Vec {
     static constexpr int kN = 16 / (int)sizeof(T);
@@ -50,32 +48,38 @@ __device__ __forceinline__ void load_vec(const __nv_bfloat16* p, Vec<__nv_bfloat
 __device__ __forceinline__ float load_x(const float* p, int64_t i) { return p[i]; }
 __device__ __forceinline__ float load_x(const __nv_bfloat16* p, int64_t i) { return __bfloat162float(p[i]); }
 
-template <class T>
+template <class T, int P>
 constexpr int64_t piece_elems() {
-    return (int64_t)kPieces * 256 * Vec<T>::kN;
+    return (int64_t)P * 256 * Vec<T>::kN;
 }
 
 // blockIdx.y = view; grid-stride over the view's pieces.
-template <class T>
+template <class T, int P>
 __global__ void __launch_bounds__(256) k_view_absmax(const T* __restrict__ x, int64_t view_elems,
                                                      uint32_t* __restrict__ amax_bits) {
     constexpr int kN = Vec<T>::kN;
     const T* xv = x + (int64_t)blockIdx.y * view_elems;
     const bool vec = (reinterpret_cast<uintptr_t>(xv) & 15) == 0;
     float m = 0.f;
-    for (int64_t e0 = (int64_t)blockIdx.x * piece_elems<T>(); e0 < view_elems;
-         e0 += (int64_t)gridDim.x * piece_elems<T>()) {
-        if (vec && e0 + piece_elems<T>() <= view_elems) {
-            Vec<T> v[kPieces];
+    for (int64_t e0 = (int64_t)blockIdx.x * piece_elems<T, P>(); e0 < view_elems;
+         e0 += (int64_t)gridDim.x * piece_elems<T, P>()) {
+        if (vec && e0 + piece_elems<T, P>() <= view_elems) {
+            Vec<T> v[P];
 #pragma unroll
-            for (int k = 0; k < kPieces; ++k) load_vec(xv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN, v[k]);
+            for (int k = 0; k < P; ++k) load_vec(xv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN, v[k]);
 #pragma unroll
-            for (int k = 0; k < kPieces; ++k)
+            for (int k = 0; k < P; ++k)
 #pragma unroll
                 for (int q = 0; q < kN; ++q) m = fmaxf(m, fabsf(v[k].x[q]));
         } else {
-            const int64_t e1 = min(view_elems, e0 + piece_elems<T>());
-            for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) m = fmaxf(m, fabsf(load_x(xv, e)));
+            const int64_t e1 = min(view_elems, e0 + piece_elems<T, P>());
+            for (int64_t e = e0 + threadIdx.x; e < e1; e += 4 * 256) {
+                float v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = e + 256 * k < e1 ? load_x(xv, e + 256 * k) : 0.f;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) m = fmaxf(m, fabsf(v[k]));
+            }
         }
     }
 #pragma unroll
@@ -105,21 +109,21 @@ __device__ __forceinline__ uint32_t e4m3_of(float x, float s) {
 // blockIdx.y = view, blockIdx.x = piece of it.  Bound by HBM (5 or 3 bytes per
 // element): 12 float32 views of 640x480x512 in 1.26 ms = 7.5 TB/s (3.14 ms with a
 // 64-bit division and a 4-byte load per element); the maximum 1.24 -> 1.05 ms.
-template <class T>
+template <class T, int P>
 __global__ void __launch_bounds__(256) k_quantize_e4m3(const T* __restrict__ x, const float* __restrict__ scales,
                                                        int64_t view_elems, uint8_t* __restrict__ q) {
     constexpr int kN = Vec<T>::kN;
     const T* xv = x + (int64_t)blockIdx.y * view_elems;
     uint8_t* qv = q + (int64_t)blockIdx.y * view_elems;
     const float s = scales[blockIdx.y];
-    const int64_t e0 = (int64_t)blockIdx.x * piece_elems<T>();
+    const int64_t e0 = (int64_t)blockIdx.x * piece_elems<T, P>();
     const bool vec = ((reinterpret_cast<uintptr_t>(xv) & 15) | (reinterpret_cast<uintptr_t>(qv) & (kN - 1))) == 0;
-    if (vec && e0 + piece_elems<T>() <= view_elems) {
-        Vec<T> v[kPieces];
+    if (vec && e0 + piece_elems<T, P>() <= view_elems) {
+        Vec<T> v[P];
 #pragma unroll
-        for (int k = 0; k < kPieces; ++k) load_vec(xv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN, v[k]);
+        for (int k = 0; k < P; ++k) load_vec(xv + e0 + (int64_t)(k * 256 + threadIdx.x) * kN, v[k]);
 #pragma unroll
-        for (int k = 0; k < kPieces; ++k) {
+        for (int k = 0; k < P; ++k) {
             uint32_t w[kN / 4];
 #pragma unroll
             for (int h = 0; h < kN / 4; ++h) {
@@ -134,9 +138,39 @@ __global__ void __launch_bounds__(256) k_quantize_e4m3(const T* __restrict__ x, 
                 *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
         }
     } else {
-        const int64_t e1 = min(view_elems, e0 + piece_elems<T>());
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) qv[e] = (uint8_t)e4m3_of(load_x(xv, e), s);
+        const int64_t e1 = min(view_elems, e0 + piece_elems<T, P>());
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += 4 * 256) {
+            float v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = e + 256 * k < e1 ? load_x(xv, e + 256 * k) : 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (e + 256 * k < e1) qv[e + 256 * k] = (uint8_t)e4m3_of(v[k], s);
+        }
     }
+}
+
+template <class T, int P>
+ludvig_status quantize(const T* x, int n_views, int64_t view_elems, uint8_t* q, float* scales, cudaStream_t st) {
+    const int64_t pieces = ceil_div(view_elems, piece_elems<T, P>());
+    LV_ARG(pieces <= 0x7fffffff, "view too large");
+    k_view_absmax<T, P><<<dim3((unsigned)std::min<int64_t>(pieces, 1024), (unsigned)n_views), 256, 0, st>>>(
+        x, view_elems, reinterpret_cast<uint32_t*>(scales));
+    LV_LAUNCH();
+    k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
+    LV_LAUNCH();
+    k_quantize_e4m3<T, P><<<dim3((unsigned)pieces, (unsigned)n_views), 256, 0, st>>>(x, scales, view_elems, q);
+    LV_LAUNCH();
+    return LUDVIG_OK;
+}
+
+// Pieces of four loads per thread where that gives the GPU a few blocks per SM; else of
+// one (3 views of 8235 bfloat16 values, the call 18 -> 14 us).
+template <class T>
+ludvig_status quantize(const T* x, int n_views, int64_t view_elems, uint8_t* q, float* scales, cudaStream_t st) {
+    return ceil_div(view_elems, piece_elems<T, 4>()) * n_views >= 4 * 152
+               ? quantize<T, 4>(x, n_views, view_elems, q, scales, st)
+               : quantize<T, 1>(x, n_views, view_elems, q, scales, st);
 }
 
 }  // namespace
@@ -156,30 +190,11 @@ extern "C" ludvig_status ludvig_fp8_quantize(const void* feats, int32_t dtype, i
     LV_ARG(((uintptr_t)q & 3) == 0, "q must be 4-byte aligned");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     LV_CUDA(cudaMemsetAsync(scales, 0, sizeof(float) * (size_t)n_views, st));
-    if (view_elems > 0) {
-        const int64_t piece = dtype == LUDVIG_F32 ? piece_elems<float>() : piece_elems<__nv_bfloat16>();
-        const int64_t pieces = ceil_div(view_elems, piece);
-        LV_ARG(pieces <= 0x7fffffff, "view too large");
-        const dim3 grid((unsigned)std::min<int64_t>(pieces, 1024), (unsigned)n_views);
-        const dim3 qgrid((unsigned)pieces, (unsigned)n_views);
-        const float* xf = static_cast<const float*>(feats);
-        const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(feats);
-        uint32_t* bits = reinterpret_cast<uint32_t*>(scales);
-        if (dtype == LUDVIG_F32)
-            k_view_absmax<float><<<grid, 256, 0, st>>>(xf, view_elems, bits);
-        else
-            k_view_absmax<__nv_bfloat16><<<grid, 256, 0, st>>>(xb, view_elems, bits);
-        LV_LAUNCH();
-        k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
-        LV_LAUNCH();
-        if (dtype == LUDVIG_F32)
-            k_quantize_e4m3<float><<<qgrid, 256, 0, st>>>(xf, scales, view_elems, q);
-        else
-            k_quantize_e4m3<__nv_bfloat16><<<qgrid, 256, 0, st>>>(xb, scales, view_elems, q);
-        LV_LAUNCH();
-    } else {
-        k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
-        LV_LAUNCH();
-    }
+    if (view_elems > 0)
+        return dtype == LUDVIG_F32
+                   ? quantize(static_cast<const float*>(feats), n_views, view_elems, q, scales, st)
+                   : quantize(static_cast<const __nv_bfloat16*>(feats), n_views, view_elems, q, scales, st);
+    k_view_scales<<<(unsigned)ceil_div(n_views, 256), 256, 0, st>>>(scales, n_views);
+    LV_LAUNCH();
     return LUDVIG_OK;
 }
