@@ -19,8 +19,9 @@
 // Bound: the FMA pipe with the embeddings' shared-memory reads close behind (n d m
 // multiply-adds, m rounded up to a multiple of 4).  500k x 512 features, 21 queries
 // and 4 phrases: 874 -> 465 us against tiles of 4 rows x 4 embeddings per thread, padded
-// to 32, and 412 with the norm's products in packed pairs behind a step's dots (before
-// them, or one by one between them, the accumulators spill: 478).  Four rows per lane at 8
+// to 32, 412 with the norm's products in packed pairs behind a step's dots (before
+// them, or one by one between them, the accumulators spill: 478), and 403 with the rows'
+// shares dealt over all SMs.  Four rows per lane at 8
 // warps per SM, and scalar instead of packed multiply-adds, measured 460 and 520 us
 // where this form took 465.
 #include <algorithm>
