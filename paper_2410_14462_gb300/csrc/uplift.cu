@@ -1595,7 +1595,9 @@ ludvig_status size_for_async(ludvig_scene* s, const std::vector<GroupViews>& gro
     }
     int nv = 1, ng = 1;
     int64_t n = 1;
+    const int ntiles = ((width + kTile - 1) / kTile) * ((height + kTile - 1) / kTile);
     for (const GroupViews& g : groups) {
+        if (tc) LV_TRY(tc_reserve_rest(s->ws, (int)g.v.size() * ntiles));
         nv = std::max(nv, (int)g.v.size());
         const int64_t npad = round_up(std::max<int64_t>(g.nmax, 1), kRadixTile);
         if ((int64_t)g.v.size() * npad > (int64_t)ng * round_up(n, kRadixTile)) {

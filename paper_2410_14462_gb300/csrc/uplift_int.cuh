@@ -135,6 +135,9 @@ ludvig_status tc_weights(const GroupLists& L, int nv, int width, int height, int
 // nitems (view, tile) items and cap chunks (allocation synchronises the device, so
 // an asynchronous call that finds them in place never waits).
 ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets);
+// The same for the tiles that the weights pass of a group of nitems may hand over
+// between its launches (nothing where the group is too small or too large for that).
+ludvig_status tc_reserve_rest(Arena& ws, int nitems);
 
 // num_v[i,:] += W^T F and den_v[i] += row sums for the group's weight rows
 // (k_aggregate_tc), view v's features at coordinate av.fview[v] of `feats`

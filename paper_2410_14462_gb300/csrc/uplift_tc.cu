@@ -136,7 +136,7 @@ constexpr int kFewTiles = 16;
 // an evenly spread scene, one channel, 0.69 -> 0.72 ms).  Larger launches have others to
 // run meanwhile: 60 views of 640x480 would go from 4.34 to 4.39 ms.
 constexpr uint32_t kHandover = 16;
-inline bool hands_over(int nitems, int sms) { return nitems < 2 * 28 * sms; }
+inline bool hands_over(int nitems, int sms) { return nitems >= kFewTiles * sms && nitems < 2 * 28 * sms; }
 
 __device__ __forceinline__ void finish_chunk(const WeightsArgs& a, int c, int rows, int next) {
     if (c >= 0 && c < a.cap) {
@@ -1915,14 +1915,23 @@ const char* const kWsPlanOff[2] = {"tc.plan_off.0", "tc.plan_off.1"};
 const char* const kWsPlan[2] = {"tc.plan.0", "tc.plan.1"};
 
 namespace {
-// The tiles that a launch of nitems may hand over.
+// The tiles that a launch of nitems may hand over: their records, then their transmittances.
 ludvig_status get_rest(Arena& ws, int nitems, int sms, WeightsArgs* w) {
-    w->limit = hands_over(nitems, sms) ? kHandover : 0xffffffffu;
+    w->limit = 0xffffffffu;
     if (!hands_over(nitems, sms)) return LUDVIG_OK;
-    LV_TRY(ws.get("tc.rest", (size_t)nitems, &w->rest));
-    return ws.get("tc.rest_t", (size_t)nitems * 256, &w->rest_t);
+    w->limit = kHandover;
+    LV_TRY(ws.get("tc.rest", (size_t)nitems * 65, &w->rest));
+    w->rest_t = reinterpret_cast<float*>(w->rest + nitems);
+    return LUDVIG_OK;
 }
 }  // namespace
+
+ludvig_status tc_reserve_rest(Arena& ws, int nitems) {
+    int sms = 0;
+    LV_TRY(sm_count(&sms));
+    WeightsArgs w;
+    return get_rest(ws, nitems, sms, &w);
+}
 
 ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets) {
     cap = std::max<int64_t>(cap, 3 * (int64_t)nitems);
@@ -1939,10 +1948,7 @@ ludvig_status tc_reserve(Arena& ws, int NT, int nitems, int64_t cap, int sets) {
         LV_TRY(ws.get(kWsPlanOff[p], sizeof(uint32_t) * ((size_t)nitems + 1), &q));
         LV_TRY(ws.get(kWsPlan[p], sizeof(int2) * (size_t)cap, &q));
     }
-    int sms = 0;
-    LV_TRY(sm_count(&sms));
-    WeightsArgs w;
-    return get_rest(ws, nitems, sms, &w);
+    return LUDVIG_OK;
 }
 
 namespace {
